@@ -14,8 +14,8 @@
 //   F   row of rho_i (each atom):         A B - 2w B' drho_i
 // rho is recomputed here from the neighbour list (no per-pair term is
 // stored).  Each warp owns shared-memory bins for all rows; its lanes add in
-// lane order, blocks are summed in block order: the gradient is bitwise
-// reproducible.
+// lane order, warps and blocks are summed in a fixed order: the gradient is
+// bitwise reproducible.
 #include "device_common.cuh"
 
 #include <cuda_runtime.h>
@@ -25,18 +25,18 @@ namespace {
 
 struct AdjDesc {
     // spline grids (FP64) of phi, f, F
-    double x0[3], h[3];
+    double x0[3], h[3], inv_h[3];
     int nint[3];       // intervals
     int row0[3];       // first bin row of each function in the bin array
     int nrows;         // total rows (sum of nint)
-    double A, w;
+    double e_ref, w;
 };
 
 __device__ __forceinline__ int adj_seg(const AdjDesc &D, int q, double x, double &t)
 {
     int k;
     if (x < D.x0[q]) k = 0;
-    else k = min((int)floor((x - D.x0[q]) / D.h[q]), D.nint[q] - 1);
+    else k = min((int)((x - D.x0[q]) * D.inv_h[q]), D.nint[q] - 1);
     t = x - (D.x0[q] + (double)k * D.h[q]);
     return k;
 }
@@ -107,153 +107,214 @@ __global__ void k_adj_g(Bufs<double> B, const double *f_ref, double *g, int n, d
     block_sums_t<1, double>(v1, partials, gridDim.x, 0);
 }
 
-// rho_i recomputed from the list, F'(rho_i), F''(rho_i), drho_i
-__global__ void k_adj_rho(Bufs<double> B, Geom G, int n, int ld, AdjDesc D, int off_f, int off_F, const double *g,
+// rho_i recomputed from the list, and drho_i.  kAdjLanes lanes share an atom
+// (columns l, l + kAdjLanes, ...; their sums meet by shuffles), so that the few
+// atoms of a configuration reach every SM: the pass is one chain of L2 trips
+// and FP64 latencies per listed pair (2,000 atoms under ncu: 82 us with a lane per atom
+// and its 26 pairs in sequence, 15 us with 8 lanes).
+constexpr int kAdjLanes = 8;
+constexpr int kAdjRhoBlock = 64;
+
+__global__ void k_adj_rho(Bufs<double> B, Geom G, int n, int ld, AdjDesc D, int off_f, const double *g,
                           double *rho_out, double *drho_out)
 {
     double h[3];
     load_h<double>(G, h);
-    const int sp = B.st->sp;
-    const double4_32a *sw = B.shadow[sp];
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const double4_32a ui = sw[p];
-    const int nn = B.nnb[p];
+    const double4_32a *sw = B.shadow[B.st->sp];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = t / kAdjLanes, l = t % kAdjLanes;
     double rho = 0.0, drho = 0.0;
-    const double gx = g[p], gy = g[(size_t)n + p], gz = g[2 * (size_t)n + p];
-    for (int k = 0; k < nn; ++k) {
-        uint32_t e = B.list[(size_t)k * ld + p];
-        int j = (int)(e & kIndexMask);
-        double4_32a uj = sw[j];
-        const Shift<double> s = entry_shift<double>(e, h);
-        double dx = (uj.x - ui.x) + s.x, dy = (uj.y - ui.y) + s.y, dz = (uj.z - ui.z) + s.z;
-        double r2 = dx * dx + dy * dy + dz * dz;
-        if (!(r2 < G.rc2)) continue;
-        double r = sqrt(r2), d1, d2;
-        rho += adj_eval(B.coef, off_f, D, 1, r, d1, d2);
-        double dr = (dx * (g[j] - gx) + dy * (g[(size_t)n + j] - gy) + dz * (g[2 * (size_t)n + j] - gz)) / r;
-        drho += d1 * dr;
+    if (p < n) {
+        const double4_32a ui = sw[p];
+        const int nn = B.nnb[p];
+        const double gx = g[p], gy = g[(size_t)n + p], gz = g[2 * (size_t)n + p];
+        for (int k = l; k < nn; k += kAdjLanes) {
+            const uint32_t e = B.list[(size_t)k * ld + p];
+            const int j = (int)(e & kIndexMask);
+            const double4_32a uj = sw[j];
+            const double hx = g[j], hy = g[(size_t)n + j], hz = g[2 * (size_t)n + j];
+            const Shift<double> s = entry_shift<double>(e, h);
+            const double dx = (uj.x - ui.x) + s.x, dy = (uj.y - ui.y) + s.y, dz = (uj.z - ui.z) + s.z;
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            if (!(r2 < G.rc2)) continue;
+            double rinv, r, d1, d2;
+            inv_r(r2, rinv, r);
+            rho += adj_eval(B.coef, off_f, D, 1, r, d1, d2);
+            drho += d1 * ((dx * (hx - gx) + dy * (hy - gy) + dz * (hz - gz)) * rinv);
+        }
     }
-    rho_out[p] = rho;
-    drho_out[p] = drho;
-    (void)off_F;
+#pragma unroll
+    for (int o = kAdjLanes / 2; o > 0; o >>= 1) {
+        rho += __shfl_xor_sync(0xffffffffu, rho, o);
+        drho += __shfl_xor_sync(0xffffffffu, drho, o);
+    }
+    if (p < n && l == 0) {
+        rho_out[p] = rho;
+        drho_out[p] = drho;
+    }
 }
 
-// Contributions of 32 atoms to the coefficient bins.  Block = kAdjWarps
-// warps over the same 32 atoms: warp w takes list columns w, w + kAdjWarps,
-// ... (and warp 0 the F rows), each into bins of its own in dynamic shared
-// memory (4 * nrows doubles per warp), added in column then lane order; the
-// block writes its warps' bins in warp order.
+// Adds each lane's four values to its row of the warp's bins (row < 0: none).
+// Lanes with the same row take turns in lane order, lanes with different rows
+// go together, so every bin sees its additions in lane order whatever the
+// other rows: a warp needs as many turns as its fullest row has lanes (about
+// 4 to 10 of 32).  All 32 lanes must call.
+__device__ __forceinline__ void add_rows(double *bins, int row, const double *c)
+{
+    const unsigned peers = __match_any_sync(0xffffffffu, row);
+    const int turn = row < 0 ? -1 : __popc(peers & ((1u << (threadIdx.x & 31u)) - 1u));
+    const int turns = __reduce_max_sync(0xffffffffu, turn) + 1;
+    for (int k = 0; k < turns; ++k) {
+        if (turn == k) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) bins[4 * row + q] += c[q];
+        }
+        __syncwarp();
+    }
+}
+
+// Contributions of kAdjAtoms atoms to the coefficient bins.  The block's
+// warps share the atoms; a warp holds them twice, lane l atom l % kAdjAtoms,
+// and takes list columns 2w + (l / kAdjAtoms), stepping by 2 x warps (warp 0
+// also the F rows).  Each warp adds into bins of its own in dynamic shared
+// memory (4 * nrows doubles); the block adds its warps' bins in warp order
+// and writes the sum.  2,000 atoms, 64 knots: 105 us with the 32 lanes adding
+// one after another (4 warps, 63 blocks), 27 us with add_rows, 8 warps and
+// 125 blocks.
+constexpr int kAdjAtoms = 16;
+
 __global__ void k_adj_accum(Bufs<double> B, Geom G, int n, int ld, AdjDesc D, int off_f, int off_F, const double *g,
                             const double *rho_in, const double *drho_in, double *block_bins)
 {
     extern __shared__ double bins_all[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    for (int r = threadIdx.x; r < warps * 4 * D.nrows; r += blockDim.x) bins_all[r] = 0.0;
     double *bins = bins_all + (size_t)warp * 4 * D.nrows;
-    for (int r = lane; r < 4 * D.nrows; r += 32) bins[r] = 0.0;
     double h[3];
     load_h<double>(G, h);
-    __syncwarp();
-    const int sp = B.st->sp;
-    const double4_32a *sw = B.shadow[sp];
-    const int p = blockIdx.x * 32 + lane;
+    const DevState *st = B.st;
+    const double A = 2.0 * ((st->e_embed + st->e_pair) - D.e_ref) / (double)n;
+    const double4_32a *sw = B.shadow[st->sp];
+    const int half = lane / kAdjAtoms;
+    const int p = blockIdx.x * kAdjAtoms + lane % kAdjAtoms;
     const bool active = p < n;
     double4_32a ui = make_double4_32a(0, 0, 0, 0);
-    double gx = 0, gy = 0, gz = 0, dF = 0, d2F = 0, drho = 0;
+    double gx = 0, gy = 0, gz = 0, dF = 0, d2F = 0, drho = 0, rho = 0;
     int nn = 0;
-    double contrib[8];
-    int row_a = -1, row_b = -1;
     if (active) {
         ui = sw[p];
         nn = B.nnb[p];
         gx = g[p]; gy = g[(size_t)n + p]; gz = g[2 * (size_t)n + p];
         drho = drho_in[p];
-        adj_eval(B.coef, off_F, D, 2, rho_in[p], dF, d2F);
-        // F row of rho_p (warp 0)
-        if (warp == 0) {
-            double bv[4], bd[4];
-            row_a = adj_rows(D, 2, rho_in[p], bv, bd);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) contrib[c] = D.A * bv[c] - 2.0 * D.w * bd[c] * drho;
-        }
+        rho = rho_in[p];
+        adj_eval(B.coef, off_F, D, 2, rho, dF, d2F);
     }
-    for (int L = 0; L < 32; ++L) {
-        if (lane == L && row_a >= 0)
+    __syncthreads();
+    double ca[4], cb[4], bv[4], bd[4];
+    if (warp == 0) {  // F row of rho_p
+        int row = -1;
+        if (active && half == 0) {
+            row = adj_rows(D, 2, rho, bv, bd);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) bins[4 * row_a + c] += contrib[c];
-        __syncwarp();
+            for (int c = 0; c < 4; ++c) ca[c] = A * bv[c] - 2.0 * D.w * bd[c] * drho;
+        }
+        add_rows(bins, row, ca);
     }
     int kmax = nn;
     for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    for (int k = warp; k < kmax; k += kAdjWarps) {
-        row_a = row_b = -1;
-        if (active && k < nn) {
-            uint32_t e = B.list[(size_t)k * ld + p];
-            int j = (int)(e & kIndexMask);
-            double4_32a uj = sw[j];
+    for (int k0 = 2 * warp; k0 < kmax; k0 += 2 * warps) {
+        const int k = k0 + half;
+        int row_a = -1, row_b = -1;
+        if (k < nn) {
+            const uint32_t e = B.list[(size_t)k * ld + p];
+            const int j = (int)(e & kIndexMask);
+            const double4_32a uj = sw[j];
+            const double hx = g[j], hy = g[(size_t)n + j], hz = g[2 * (size_t)n + j];
             const Shift<double> s = entry_shift<double>(e, h);
-            double dx = (uj.x - ui.x) + s.x, dy = (uj.y - ui.y) + s.y, dz = (uj.z - ui.z) + s.z;
-            double r2 = dx * dx + dy * dy + dz * dz;
+            const double dx = (uj.x - ui.x) + s.x, dy = (uj.y - ui.y) + s.y, dz = (uj.z - ui.z) + s.z;
+            const double r2 = dx * dx + dy * dy + dz * dz;
             if (r2 < G.rc2) {
-                double r = sqrt(r2);
-                double dr = (dx * (g[j] - gx) + dy * (g[(size_t)n + j] - gy) + dz * (g[2 * (size_t)n + j] - gz)) / r;
-                double bv[4], bd[4];
+                double rinv, r;
+                inv_r(r2, rinv, r);
+                const double dr = (dx * (hx - gx) + dy * (hy - gy) + dz * (hz - gz)) * rinv;
                 row_a = adj_rows(D, 0, r, bv, bd);  // phi
 #pragma unroll
-                for (int c = 0; c < 4; ++c) contrib[c] = 0.5 * D.A * bv[c] - D.w * bd[c] * dr;
+                for (int c = 0; c < 4; ++c) ca[c] = 0.5 * A * bv[c] - D.w * bd[c] * dr;
                 row_b = adj_rows(D, 1, r, bv, bd);  // f
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    contrib[4 + c] = D.A * dF * bv[c] - 2.0 * D.w * (d2F * drho * bv[c] + dF * bd[c] * dr);
+                    cb[c] = A * dF * bv[c] - 2.0 * D.w * (d2F * drho * bv[c] + dF * bd[c] * dr);
             }
         }
-        for (int L = 0; L < 32; ++L) {
-            if (lane == L && row_a >= 0) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) bins[4 * row_a + c] += contrib[c];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) bins[4 * row_b + c] += contrib[4 + c];
-            }
-            __syncwarp();
-        }
+        add_rows(bins, row_a, ca);
+        add_rows(bins, row_b, cb);
     }
-    for (int r = lane; r < 4 * D.nrows; r += 32)
-        block_bins[((size_t)blockIdx.x * kAdjWarps + warp) * 4 * D.nrows + r] = bins[r];
+    __syncthreads();
+    for (int r = threadIdx.x; r < 4 * D.nrows; r += blockDim.x) {
+        double s = 0.0;
+        for (int w = 0; w < warps; ++w) s += bins_all[(size_t)w * 4 * D.nrows + r];
+        block_bins[(size_t)blockIdx.x * 4 * D.nrows + r] = s;
+    }
 }
 
-// Sum the block bins in block order (one thread per coefficient), and the
-// |g|^2 block partials.
+// Sum of the blocks' bins, in a fixed order: 32 coefficients per block of
+// 32 x kFinishParts threads, part y taking block bins y, y + kFinishParts, ...
+// (four loads in flight), the parts added in order.  Also the |g|^2 block
+// partials (block 0).  One thread per coefficient walked all the bins in
+// sequence: 42 us at 2,000 atoms, against 5 us.
+constexpr int kFinishParts = 16;
+
 __global__ void k_adj_finish(const double *block_bins, int nblocks, int nrows, const double *partials_g, int nb_g,
                              double *coef_grad, double *sq_out)
 {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < 4 * nrows; r += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += block_bins[(size_t)b * 4 * nrows + r];
-        coef_grad[r] = s;
+    __shared__ double sm[kFinishParts][33];
+    const int x = threadIdx.x, y = threadIdx.y, r = blockIdx.x * 32 + x;
+    double s = 0.0;
+    if (r < 4 * nrows) {
+        const double *b = block_bins + r;
+        const size_t step = 4 * (size_t)nrows;
+#pragma unroll 4
+        for (int k = y; k < nblocks; k += kFinishParts) s += b[(size_t)k * step];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nb_g; ++b) s += partials_g[b];
-        *sq_out = s;
+    sm[y][x] = s;
+    __syncthreads();
+    if (y == 0 && r < 4 * nrows) {
+        double t = 0.0;
+        for (int k = 0; k < kFinishParts; ++k) t += sm[k][x];
+        coef_grad[r] = t;
+    }
+    if (blockIdx.x == 0 && y == 1) {
+        double q = 0.0;
+        for (int b = x; b < nb_g; b += 32) q += partials_g[b];
+        q = warp_sum_d(q);
+        if (x == 0) *sq_out = q;
     }
 }
 
 // knot gradient: for knot q of function fn, sum over that function's
 // coefficient rows of M[row][q] * coef_grad[row] (M stored transposed:
-// Mt[q][row] over the function's 4*nint coefficients, fixed order).
+// Mt[q][row] over the function's 4*nint coefficients), a warp per knot: lane l
+// rows l, l + 32, ..., the lanes' sums meeting by shuffles (47 us with a
+// thread per knot at 3 x 64 knots, 7 us so).
 __global__ void k_adj_knots(const double *coef_grad, const double *Mt, int nknots_total, const int *knot_func,
                             const int *func_coef0, const int *func_ncoef, const long long *knot_mt0,
                             double *knot_grad)
 {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nknots_total) return;
-    int fn = knot_func[q];
+    const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (q >= nknots_total) return;  // the same for a warp's lanes
+    const int fn = knot_func[q];
     const double *m = Mt + knot_mt0[q];
     const double *cg = coef_grad + func_coef0[fn];
     double s = 0.0;
-    for (int r = 0; r < func_ncoef[fn]; ++r) s += m[r] * cg[r];
-    knot_grad[q] = s;
+    for (int r = lane; r < func_ncoef[fn]; r += 32) s += m[r] * cg[r];
+    s = warp_sum_d(s);
+    if (lane == 0) knot_grad[q] = s;
 }
+
+// Warps of a block of the accumulation: as many as share 16 atoms' columns
+// usefully (8) while their bins fit 96 KB, which lets two blocks share an SM;
+// 4 for larger tables (up to the limit the host checks).
+int adjoint_warps(int nrows) { return 8 * sizeof(double) * 4 * (size_t)nrows <= 96 * 1024 ? 8 : kAdjWarps; }
 
 }  // namespace
 
@@ -264,39 +325,44 @@ int launch_adjoint(const Bufs<double> &B, const Geom &G, const Launch &L, const 
     for (int q = 0; q < 3; ++q) {
         D.x0[q] = a.x0[q];
         D.h[q] = a.h[q];
+        D.inv_h[q] = 1.0 / a.h[q];
         D.nint[q] = a.nint[q];
         D.row0[q] = row;
         row += a.nint[q];
     }
     D.nrows = row;
-    D.A = a.A;
+    D.e_ref = a.e_ref;
     D.w = a.w;
     const int n = L.n;
     const int nb = blocks_for(n, 256);
     k_adj_g<<<nb, 256, 0, L.stream>>>(B, a.f_ref, a.g, n, a.partials_g);
-    // one warp per block: the few atoms of a force-matching configuration
-    // spread over as many SMs' FP64 pipes as they can fill
-    k_adj_rho<<<blocks_for(n, 32), 32, 0, L.stream>>>(B, G, n, L.ld, D, a.off_f, a.off_F, a.g, a.rho, a.drho);
-    const int nw = blocks_for(n, 32);
+    k_adj_rho<<<blocks_for((long long)n * kAdjLanes, kAdjRhoBlock), kAdjRhoBlock, 0, L.stream>>>(
+        B, G, n, L.ld, D, a.off_f, a.g, a.rho, a.drho);
+    const int nw = adjoint_blocks(n), warps = adjoint_warps(D.nrows);
     const size_t smem = adjoint_smem_bytes(D.nrows);
-    k_adj_accum<<<nw, 32 * kAdjWarps, smem, L.stream>>>(B, G, n, L.ld, D, a.off_f, a.off_F, a.g, a.rho, a.drho,
-                                                        a.block_bins);
-    k_adj_finish<<<blocks_for(4 * D.nrows, 256), 256, 0, L.stream>>>(a.block_bins, nw * kAdjWarps, D.nrows,
-                                                                      a.partials_g, nb, a.coef_grad, a.sq);
+    k_adj_accum<<<nw, 32 * warps, smem, L.stream>>>(B, G, n, L.ld, D, a.off_f, a.off_F, a.g, a.rho, a.drho,
+                                                    a.block_bins);
+    k_adj_finish<<<blocks_for(4 * D.nrows, 32), dim3(32, kFinishParts), 0, L.stream>>>(
+        a.block_bins, nw, D.nrows, a.partials_g, nb, a.coef_grad, a.sq);
     int launched = 4;
     if (a.knot_grad) {
-        k_adj_knots<<<blocks_for(a.nknots_total, 128), 128, 0, L.stream>>>(
+        k_adj_knots<<<blocks_for((long long)a.nknots_total * 32, 256), 256, 0, L.stream>>>(
             a.coef_grad, a.Mt, a.nknots_total, a.knot_func, a.func_coef0, a.func_ncoef, a.knot_mt0, a.knot_grad);
         ++launched;
     }
     return launched;
 }
 
-size_t adjoint_smem_bytes(int nrows) { return sizeof(double) * 4 * (size_t)nrows * kAdjWarps; }
+size_t adjoint_smem_bytes(int nrows) { return sizeof(double) * 4 * (size_t)nrows * adjoint_warps(nrows); }
 
-cudaError_t allow_adjoint_smem(size_t bytes)
+int adjoint_blocks(int n) { return blocks_for(n, kAdjAtoms); }
+
+// The limit belongs to the kernel, not to a context: always the largest that
+// the host admits, so that contexts of different tables do not lower it for
+// each other.
+cudaError_t allow_adjoint_smem()
 {
-    return cudaFuncSetAttribute(k_adj_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return cudaFuncSetAttribute(k_adj_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjMaxSmem);
 }
 
 }  // namespace eammd

@@ -97,6 +97,7 @@ struct md_ctx {
     int *adj_knot_func = nullptr, *adj_func_coef0 = nullptr, *adj_func_ncoef = nullptr;
     long long *adj_knot_mt0 = nullptr;
     int adj_nrows = 0, adj_nknots = 0;
+    double *adj_host = nullptr;   // pinned: |g|^2, then the knot gradient
     // persistent step launch (md_step as one cooperative kernel)
     PersistScratch *ps = nullptr;
     int persist_tpa = 0, persist_grid = 0;  // 0: graph path
@@ -902,7 +903,7 @@ md_status set_potential_impl(md_ctx *ctx, const md_potential *pot)
 // Adjoint workspace and the transposed spline basis maps of phi, f, F.
 md_status adjoint_setup(md_ctx *ctx)
 {
-    if (ctx->adj_g) return MD_OK;
+    if (ctx->adj_host) return MD_OK;
     const size_t n = (size_t)ctx->n;
     const md_spline *fs[3] = {&ctx->shapes[2], &ctx->shapes[1], &ctx->shapes[0]};  // phi, f, F
     int nrows = 0, nknots = 0;
@@ -910,8 +911,8 @@ md_status adjoint_setup(md_ctx *ctx)
         nrows += sp->n - 1;
         nknots += sp->n;
     }
-    if (adjoint_smem_bytes(nrows) > 200 * 1024) return ctx->fail(MD_ERR_CAPACITY, "too many spline intervals for the adjoint bins");
-    CK(allow_adjoint_smem(adjoint_smem_bytes(nrows)));
+    if (adjoint_smem_bytes(nrows) > kAdjMaxSmem) return ctx->fail(MD_ERR_CAPACITY, "too many spline intervals for the adjoint bins");
+    CK(allow_adjoint_smem());
     std::vector<double> Mt;
     std::vector<int> knot_func, coef0(3), ncoef(3);
     std::vector<long long> mt0;
@@ -936,17 +937,14 @@ md_status adjoint_setup(md_ctx *ctx)
             Mt.insert(Mt.end(), rows.begin(), rows.end());
         }
     }
-    const int nw = (int)((n + 31) / 32), nb = (int)((n + 255) / 256);
+    const int nw = adjoint_blocks((int)n), nb = (int)((n + 255) / 256);
     bool ok = alloc_n(ctx, ctx->adj_g, 3 * n) && alloc_n(ctx, ctx->adj_rho, n) && alloc_n(ctx, ctx->adj_drho, n) &&
-              alloc_n(ctx, ctx->adj_bins, (size_t)nw * kAdjWarps * 4 * nrows) && alloc_n(ctx, ctx->adj_pg, (size_t)nb) &&
+              alloc_n(ctx, ctx->adj_bins, (size_t)nw * 4 * nrows) && alloc_n(ctx, ctx->adj_pg, (size_t)nb) &&
               alloc_n(ctx, ctx->adj_cg, (size_t)4 * nrows) && alloc_n(ctx, ctx->adj_sq, 1) &&
               alloc_n(ctx, ctx->adj_Mt, Mt.size()) && alloc_n(ctx, ctx->adj_kg, (size_t)nknots) &&
               alloc_n(ctx, ctx->adj_knot_func, (size_t)nknots) && alloc_n(ctx, ctx->adj_func_coef0, 3) &&
               alloc_n(ctx, ctx->adj_func_ncoef, 3) && alloc_n(ctx, ctx->adj_knot_mt0, (size_t)nknots);
-    if (!ok) {
-        ctx->adj_g = nullptr;
-        return ctx->fail(MD_ERR_OOM, "adjoint workspace");
-    }
+    if (!ok) return ctx->fail(MD_ERR_OOM, "adjoint workspace");
     CK(cudaMemcpy(ctx->adj_Mt, Mt.data(), Mt.size() * sizeof(double), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->adj_knot_func, knot_func.data(), knot_func.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->adj_func_coef0, coef0.data(), 3 * sizeof(int), cudaMemcpyHostToDevice));
@@ -954,15 +952,13 @@ md_status adjoint_setup(md_ctx *ctx)
     CK(cudaMemcpy(ctx->adj_knot_mt0, mt0.data(), mt0.size() * sizeof(long long), cudaMemcpyHostToDevice));
     ctx->adj_nrows = nrows;
     ctx->adj_nknots = nknots;
+    CK(cudaMallocHost((void **)&ctx->adj_host, sizeof(double) * ((size_t)nknots + 1)));
     return MD_OK;
 }
 
 md_status force_match_impl(md_ctx *ctx, const double *f_ref, double e_ref, double w, double *loss, double *grad)
 {
-    md_status rc = check_device_errors(ctx);
-    if (rc != MD_OK) return rc;
-    const double E = ctx->st_host->e_embed + ctx->st_host->e_pair;
-    rc = adjoint_setup(ctx);
+    md_status rc = adjoint_setup(ctx);
     if (rc != MD_OK) return rc;
     const size_t n = (size_t)ctx->n;
     CK(cudaMemcpyAsync(ctx->stage, f_ref, 3 * n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
@@ -976,7 +972,7 @@ md_status force_match_impl(md_ctx *ctx, const double *f_ref, double e_ref, doubl
     }
     a.off_f = ctx->off_f0;
     a.off_F = ctx->off_F0;
-    a.A = 2.0 * (E - e_ref) / (double)n;
+    a.e_ref = e_ref;
     a.w = w;
     a.f_ref = ctx->stage;
     a.g = ctx->adj_g;
@@ -996,12 +992,19 @@ md_status force_match_impl(md_ctx *ctx, const double *f_ref, double e_ref, doubl
     Launch L = ctx->L;
     ctx->fixed_launches += launch_adjoint(ctx->Bd, ctx->G, L, a);
     CK(cudaGetLastError());
-    double sq = 0.0;
-    CK(cudaMemcpyAsync(&sq, ctx->adj_sq, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    // one wait for the energy, the error flags, |g|^2 and the gradient: the
+    // kernels take the energy from the device state
+    double *out = ctx->adj_host;
+    CK(cudaMemcpyAsync(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(out, ctx->adj_sq, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if (grad)
-        CK(cudaMemcpyAsync(grad, ctx->adj_kg, sizeof(double) * (size_t)ctx->adj_nknots, cudaMemcpyDeviceToHost,
+        CK(cudaMemcpyAsync(out + 1, ctx->adj_kg, sizeof(double) * (size_t)ctx->adj_nknots, cudaMemcpyDeviceToHost,
                            ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    rc = state_errors(ctx);
+    if (rc != MD_OK) return rc;
+    const double E = ctx->st_host->e_embed + ctx->st_host->e_pair, sq = out[0];
+    if (grad) memcpy(grad, out + 1, sizeof(double) * (size_t)ctx->adj_nknots);
     if (loss) *loss = (E - e_ref) * (E - e_ref) / (double)n + w * sq;
     return MD_OK;
 }
@@ -1483,6 +1486,7 @@ void md_destroy(md_ctx *ctx)
         if (ctx->Bf.tex_shadow[s]) cudaDestroyTextureObject((cudaTextureObject_t)ctx->Bf.tex_shadow[s]);
     dfree_all(ctx);
     if (ctx->st_host) cudaFreeHost(ctx->st_host);
+    if (ctx->adj_host) cudaFreeHost(ctx->adj_host);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->body_stream) cudaStreamDestroy(ctx->body_stream);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);

@@ -221,10 +221,10 @@ struct AdjointArgs {
     double x0[3], h[3];
     int nint[3];
     int off_f, off_F;       // coefficient offsets of f and F in B.coef
-    double A, w;
+    double e_ref, w;
     const double *f_ref;    // n*3, caller order (device)
     double *g, *rho, *drho; // 3n, n, n
-    double *block_bins;     // nblocks_warp * 4 * nrows
+    double *block_bins;     // adjoint_blocks(n) * 4 * nrows
     double *partials_g;     // >= blocks of k_adj_g
     double *coef_grad;      // 4 * nrows
     double *sq;             // 1
@@ -237,9 +237,11 @@ struct AdjointArgs {
 
 int launch_adjoint(const Bufs<double> &B, const Geom &G, const Launch &L, const AdjointArgs &a);
 size_t adjoint_smem_bytes(int nrows);
-// Permits `bytes` of dynamic shared memory to the adjoint accumulation.
-cudaError_t allow_adjoint_smem(size_t bytes);
-// Warps that share the 32 atoms of one block of the adjoint accumulation.
+int adjoint_blocks(int n);  // blocks of the accumulation
+// Permits kAdjMaxSmem bytes of dynamic shared memory to the adjoint accumulation.
+constexpr size_t kAdjMaxSmem = 200 * 1024;
+cudaError_t allow_adjoint_smem();
+// Fewest warps of a block of the adjoint accumulation, whose bins have to fit.
 constexpr int kAdjWarps = 4;
 
 }  // namespace eammd
