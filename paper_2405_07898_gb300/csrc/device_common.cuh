@@ -20,8 +20,14 @@ template <> __device__ __forceinline__ double4_32a mk4<double>(double x, double 
     return make_double4_32a(x, y, z, w);
 }
 
-// 1/r and r from r^2: one MUFU reciprocal square root in FP32, IEEE sqrt and
-// division in FP64.
+// 1/r and r from r^2.  FP32: one MUFU reciprocal square root.  FP64: the
+// hardware's approximate reciprocal square root y (about 20 bits) and one
+// third-order step of y -> 1/sqrt(x) in the residual e = 1 - x y^2,
+//   (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + O(e^3),
+// applied to y and to a = x y, which give 1/r and r together to about one
+// rounding: 6 FP64 operations (5 where 1/r is not used) where an IEEE square
+// root and a division take about 18.  The FP64 pipe bounds the FP64 pair
+// passes (2 operations per clock and SM).  r2 = 0 gives NaN.
 __device__ __forceinline__ void inv_r(float r2, float &rinv, float &r)
 {
     rinv = rsqrtf(r2);
@@ -29,8 +35,13 @@ __device__ __forceinline__ void inv_r(float r2, float &rinv, float &r)
 }
 __device__ __forceinline__ void inv_r(double r2, double &rinv, double &r)
 {
-    r = sqrt(r2);
-    rinv = 1.0 / r;
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    const double a = r2 * y;
+    const double e = fma(-a, y, 1.0);
+    const double p = fma(0.375, e, 0.5) * e;
+    rinv = fma(y, p, y);
+    r = fma(a, p, a);
 }
 
 // Cubic spline in r on a table that covers [x0, x_end] with x0 <= 0 and
@@ -88,6 +99,31 @@ __device__ __forceinline__ int segment(const SplineDesc<R> &s, R x, R &t)
     int k = min((int)u, s.nint - 1);
     R kf = (R)k;
     t = fma(-kf, s.h_lo, fma(-kf, s.h_hi, x - s.x0));
+    return k;
+}
+
+// The same for the fused one-type tables (x0 <= 0 <= x < x_end, fewer than
+// 2^22 intervals): the interval comes from adding u = (x - x0)/h rounded down
+// to a power of two whose unit in the last place is 1 (2^23 in FP32, 2^52 in
+// FP64), where the low bits of the sum are floor(u); subtracting the power
+// again gives floor(u) as a number.  Two additions stand for the conversions
+// to integer and back, which run at an eighth of the FP32 rate (FP32) or on
+// the narrow FP64 pipe.  The bits are compared as unsigned integers, so that
+// a NaN takes the last interval.
+__device__ __forceinline__ int segment_fused(const SplineDesc<float> &s, float x, float &t)
+{
+    const float xr = x - s.x0;
+    const unsigned m = min(__float_as_uint(__fadd_rd(xr * s.inv_h, 0x1p23f)), 0x4B000000u + (unsigned)(s.nint - 1));
+    const float kf = __uint_as_float(m) - 0x1p23f;
+    t = fmaf(-kf, s.h_lo, fmaf(-kf, s.h_hi, xr));
+    return (int)(m - 0x4B000000u);
+}
+__device__ __forceinline__ int segment_fused(const SplineDesc<double> &s, double x, double &t)
+{
+    const double xr = x - s.x0;
+    const int k = (int)min((unsigned)__double2loint(__fma_rd(xr, s.inv_h, 0x1p52)), (unsigned)(s.nint - 1));
+    const double kf = __hiloint2double(0x43300000, k) - 0x1p52;
+    t = fma(-kf, s.h_hi, xr);  // h_lo is zero in FP64
     return k;
 }
 

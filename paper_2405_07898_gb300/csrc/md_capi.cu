@@ -246,7 +246,8 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
     if (!ok) return false;
     B.coef = coef;
     B.coef2 = coef2;
-    B.coef_f = tables.fused ? coef2 + 2 * (size_t)tables.fphi.nint : coef2;
+    B.coef_d = tables.fused ? coef2 + 2 * (size_t)tables.fphi.nint : coef2;
+    B.coef_f = tables.fused ? coef2 + 4 * (size_t)tables.fphi.nint : coef2;
     B.tables = tab;
     B.st = ctx->st;
     auto upload = [](R4 *dst_dev, const std::vector<double> &src) -> bool {
@@ -646,6 +647,18 @@ md_status build_tables(md_ctx *ctx, const md_potential *pot, std::vector<double>
             for (int c = 0; c < 4; ++c) rows2.push_back(rows[4 * ((size_t)tab.f[0].offset + k) + c]);
             for (int c = 0; c < 4; ++c) rows2.push_back(rows[4 * ((size_t)tab.phi[0].offset + k) + c]);
         }
+        // then the rows of the derivatives: b, 2c, 3d of f and of phi, the
+        // products rounded as the kernels would (3d of the rounded d)
+        for (int k = 0; k < f0.n - 1; ++k) {
+            for (const auto &d : {tab.f[0], tab.phi[0]}) {
+                const double *c = &rows[4 * ((size_t)d.offset + k)];
+                rows2.push_back(c[1]);
+                rows2.push_back(2.0 * c[2]);
+                rows2.push_back((double)((R)3 * (R)c[3]));
+            }
+            rows2.push_back(0.0);
+            rows2.push_back(0.0);
+        }
         // then the f rows alone, for the density pass: twice as many
         // intervals per cache line as in the interleaved rows
         for (int k = 0; k < f0.n - 1; ++k)
@@ -719,7 +732,7 @@ md_status autotune(md_ctx *ctx)
     // wave of blocks on the GPU
     std::vector<PassSched> cand;
     for (int t : {1, 2})
-        for (int b : {256, 224, 192, 160, 128, 96, 64}) cand.push_back({t, b});
+        for (int b : {128, 256, 192, 224, 160, 96, 64}) cand.push_back({t, b});
     cand.push_back({4, 256});
     cand.push_back({8, 256});
     const int nc = (int)cand.size();
@@ -762,11 +775,14 @@ md_status autotune(md_ctx *ctx)
         }
     }
     CK(cudaMemcpy(ctx->st, &saved, sizeof(DevState), cudaMemcpyHostToDevice));
-    // candidates in order of preference: a later one must win by 3%
+    // candidates in order of preference: a later one must win by 1.5%, about
+    // three times what the minimum over the rounds varies by (the block sizes
+    // of one lane per atom differ by up to 4%: force pass, 799,496 atoms,
+    // 84.9 us with 128 threads, 86.8 with 192, 88.4 with 256)
     int cd = 0, cf = 0;
     for (int ci = 1; ci < nc; ++ci) {
-        if (best_d[ci] < 0.97f * best_d[cd]) cd = ci;
-        if (best_f[ci] < 0.97f * best_f[cf]) cf = ci;
+        if (best_d[ci] < 0.985f * best_d[cd]) cd = ci;
+        if (best_f[ci] < 0.985f * best_f[cf]) cf = ci;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1017,9 +1033,9 @@ md_status create_impl(md_ctx *ctx, const double *pos, const double *vel, const i
     Tables<R> tab;
     md_status trc = build_tables<R>(ctx, pot, rows, rows2, tab);
     if (trc != MD_OK) return trc;
-    ctx->L.multi = tab.fused ? 0 : 1;
+    ctx->L.multi = tab.fused && tab.fphi.nint <= kMaxFusedIntervals ? 0 : 1;
     ctx->L.nint_fused = tab.fused ? tab.fphi.nint : 0;
-    if (ctx->opt.half_list && (ctx->precision != MD_PRECISION_MIXED || ctx->L.multi))
+    if (ctx->opt.half_list && (ctx->precision != MD_PRECISION_MIXED || !tab.fused))
         return ctx->fail(MD_ERR_ARG, "half_list takes mixed precision and one atom type whose f and phi share a knot grid");
     ctx->L.half = ctx->opt.half_list ? 1 : 0;
     ctx->shapes.clear();

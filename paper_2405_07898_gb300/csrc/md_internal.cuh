@@ -151,7 +151,9 @@ struct Bufs {
     DevState *st;
     const R4 *coef;
     const R4 *coef2;     // fused f | phi rows (single-type fast path)
-    const R4 *coef_f;    // the f rows alone (coef2 + 2 nint), read by the density pass
+    const R4 *coef_f;    // the f rows alone (coef2 + 4 nint), read by the density pass
+    const R4 *coef_d;    // rows (f': b, 2c, 3d; phi': b, 2c, 3d; 0, 0) (coef2 + 2 nint), read by the
+                         // force pass when it forms no energies
     const Tables<R> *tables;
 };
 

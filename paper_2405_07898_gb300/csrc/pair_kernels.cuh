@@ -36,6 +36,48 @@ __device__ __forceinline__ PairIn<R> pair_vector(const typename V4<R>::T &ui, co
     return p;
 }
 
+// Pair vector and squared distance in FP64 from the atom's own coordinates
+// shifted into the neighbour's cell (one addition per component less than
+// u_j - u_i + shift; the three candidates per axis are formed once per atom).
+template <class R> struct Own {
+    typename V4<R>::T u;
+    R h[3];
+    __device__ __forceinline__ Own(const typename V4<R>::T &ui, const R (&hh)[3]) : u(ui), h{hh[0], hh[1], hh[2]} {}
+    __device__ __forceinline__ PairIn<R> to(const typename V4<R>::T &uj, uint32_t e) const
+    {
+        return pair_vector<R>(u, uj, entry_shift<R>(e, h));
+    }
+};
+template <> struct Own<double> {
+    double x[3], y[3], z[3];
+    __device__ __forceinline__ Own(const double4_32a &u, const double (&h)[3])
+        : x{u.x + h[0], u.x, u.x - h[0]}, y{u.y + h[1], u.y, u.y - h[1]}, z{u.z + h[2], u.z, u.z - h[2]}
+    {
+    }
+    static __device__ __forceinline__ double pick(const double (&v)[3], uint32_t t)
+    {
+        return t == 1u ? v[1] : (t == 0u ? v[0] : v[2]);
+    }
+    __device__ __forceinline__ PairIn<double> to(const double4_32a &uj, uint32_t e) const
+    {
+        const uint32_t c = e >> kCodeShift;
+        PairIn<double> p;
+        p.dx = uj.x - pick(x, c & 3u);
+        p.dy = uj.y - pick(y, (c >> 2) & 3u);
+        p.dz = uj.z - pick(z, c >> 4);
+        p.r2 = fma(p.dz, p.dz, fma(p.dy, p.dy, p.dx * p.dx));
+        return p;
+    }
+};
+
+// r2 < rc2 for a non-negative r2 (or NaN: false).  Non-negative doubles order
+// as their bits, which keeps the comparison off the FP64 pipe.
+__device__ __forceinline__ bool within(float r2, float rc2) { return r2 < rc2; }
+__device__ __forceinline__ bool within(double r2, double rc2)
+{
+    return (unsigned long long)__double_as_longlong(r2) < (unsigned long long)__double_as_longlong(rc2);
+}
+
 // Both 16-byte halves of a 32-byte fused row with one 256-bit load.
 template <class R>
 __device__ __forceinline__ void load_row2(const typename V4<R>::T *row, typename V4<R>::T &a, typename V4<R>::T &b);
@@ -80,15 +122,25 @@ struct TexFetch {
 // Where the spline rows of the one-type path are read from: coef2 in device
 // memory (row 2k: f, row 2k+1: phi, both in one 32-byte load); the density
 // pass reads the f rows alone from coef_f, where a 128-byte line holds eight
-// intervals instead of four.
+// intervals instead of four; the force pass without energies reads coef_d,
+// the rows of f' and phi' (b, 2c, 3d of each, six of a row's eight words).
 template <class R>
 struct TabGlobal {
     const typename V4<R>::T *coef2;
     const typename V4<R>::T *coef_f;  // f rows alone: more intervals per cache line
+    const typename V4<R>::T *coef_d;  // f' and phi' rows
     __device__ __forceinline__ typename V4<R>::T f(int kk) const { return coef_f[kk]; }
     __device__ __forceinline__ void fphi(int kk, typename V4<R>::T &cf, typename V4<R>::T &cp) const
     {
         load_row2<R>(coef2 + 2 * kk, cf, cp);
+    }
+    // f' and phi' at t
+    __device__ __forceinline__ void slopes(int kk, R t, R &fd, R &pd) const
+    {
+        typename V4<R>::T a, b;
+        load_row2<R>(coef_d + 2 * kk, a, b);
+        fd = fma(t, fma(t, a.z, a.y), a.x);
+        pd = fma(t, fma(t, b.y, b.x), a.w);
     }
 };
 // Where list column k of the lane's atom is read from.
@@ -118,6 +170,7 @@ __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R r
     using R4 = typename V4<R>::T;
     const Tables<R> &T = *B.tables;
     const SplineDesc<R> g = MULTI ? T.f[0] : T.fphi;
+    const Own<R> own(ui, h);
     R rho = (R)0;
     (void)cap;
     const int nn = *nnb_i;
@@ -132,8 +185,8 @@ __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R r
         for (int q = 0; q < U; ++q) u[q] = fetch(q == 0 || k + q * TPA < nn ? e[q] : e[0]);
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            const PairIn<R> p = pair_vector<R>(ui, u[q], entry_shift<R>(e[q], h));
-            if ((q == 0 || k + q * TPA < nn) && p.r2 < rc2) {
+            const PairIn<R> p = own.to(u[q], e[q]);
+            if ((q == 0 || k + q * TPA < nn) && within(p.r2, rc2)) {
                 R rinv, r;
                 inv_r(p.r2, rinv, r);
                 if (MULTI) {
@@ -143,7 +196,7 @@ __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R r
                     rho += val;
                 } else {
                     R t;
-                    const int kk = segment(g, r, t);
+                    const int kk = segment_fused(g, r, t);
                     const R4 c = tab.f(kk);
                     rho += fma(t, fma(t, fma(t, c.w, c.z), c.y), c.x);
                 }
@@ -180,6 +233,7 @@ __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, co
     const Tables<R> &T = *B.tables;
     const SplineDesc<R> g = T.fphi;
     const R Fpi = ui.w;
+    const Own<R> own(ui, h);
     constexpr int W = U * TPA;  // columns per round
     uint32_t e[U], en[U];
     R4 u[U];
@@ -202,8 +256,8 @@ __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, co
         for (int q = 0; q < U; ++q) e2[q] = (k1 + W + q * TPA < nn) ? list(k1 + W + q * TPA) : 0u;
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            const PairIn<R> p = pair_vector<R>(ui, u[q], entry_shift<R>(e[q], h));
-            if ((q == 0 || k + q * TPA < nn) && p.r2 < rc2) {
+            const PairIn<R> p = own.to(u[q], e[q]);
+            if ((q == 0 || k + q * TPA < nn) && within(p.r2, rc2)) {
                 R rinv, r;
                 inv_r(p.r2, rinv, r);
                 const R Fpj = u[q].w;
@@ -216,13 +270,18 @@ __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, co
                     fdi = (tj == ti) ? fdj : spline_r_der(T.f[ti], B.coef, r);
                 } else {
                     R t;
-                    const int kk = segment(g, r, t);
-                    R4 cf, cp;
-                    tab.fphi(kk, cf, cp);
-                    fdj = fma(t, fma(t, (R)3 * cf.w, (R)2 * cf.z), cf.y);
+                    const int kk = segment_fused(g, r, t);
+                    if (ENERGY) {
+                        R4 cf, cp;
+                        tab.fphi(kk, cf, cp);
+                        fdj = fma(t, fma(t, (R)3 * cf.w, (R)2 * cf.z), cf.y);
+                        phd = fma(t, fma(t, (R)3 * cp.w, (R)2 * cp.z), cp.y);
+                        phv = fma(t, fma(t, fma(t, cp.w, cp.z), cp.y), cp.x);
+                    } else {
+                        tab.slopes(kk, t, fdj, phd);
+                        phv = (R)0;
+                    }
                     fdi = fdj;
-                    phd = fma(t, fma(t, (R)3 * cp.w, (R)2 * cp.z), cp.y);
-                    phv = ENERGY ? fma(t, fma(t, fma(t, cp.w, cp.z), cp.y), cp.x) : (R)0;
                 }
                 const R sij = fma(Fpj, fdi, fma(Fpi, fdj, phd));
                 const R sr = sij * rinv;
@@ -370,11 +429,11 @@ __global__ void __launch_bounds__(256) k_density(Bufs<R> B, Geom G, Launch L)
             rho = density_lane<R, MULTI, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, sw[i],
                                                  ListGlobal{B.list + i, L.ld},
                                                  TexFetch{(cudaTextureObject_t)B.tex_shadow[sp]},
-                                                 TabGlobal<R>{B.coef2, B.coef_f});
+                                                 TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
         else
             rho = density_lane<R, MULTI, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, sw[i],
                                                  ListGlobal{B.list + i, L.ld}, GlobalFetch<R>{sw},
-                                                 TabGlobal<R>{B.coef2, B.coef_f});
+                                                 TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
     }
     rho = lane_sum<TPA>(rho);
     R e_embed = (R)0;
@@ -406,7 +465,7 @@ __global__ void __launch_bounds__(256) k_force(Bufs<R> B, Geom G, Launch L)
     R e7[7] = {0, 0, 0, 0, 0, 0, 0};
     if (active)
         force_lane<R, MULTI, ENERGY, TPA, U>(B, L, h, rc2, s, B.nnb + i, l, ti, sw[i], ListGlobal{B.list + i, L.ld},
-                                             GlobalFetch<R>{sw}, f, e7, TabGlobal<R>{B.coef2, B.coef_f});
+                                             GlobalFetch<R>{sw}, f, e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
 #pragma unroll
     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
     double ke = 0.0;
