@@ -44,6 +44,8 @@ __host__ __device__ constexpr uint32_t list_entry(uint32_t q, int dx, int dy, in
 {
     return q | ((uint32_t)((dx + 1) | ((dy + 1) << 2) | ((dz + 1) << 4)) << kCodeShift);
 }
+// Largest fused table of the full-list pair passes (segment_fused).
+constexpr int kMaxFusedIntervals = 1 << 22;
 constexpr int kScanBlock = 1024;
 constexpr int kEnergySlots = 10;  // embed, pair, ke, virial xx yy zz xy xz yz, spare
 constexpr double kAccel = 9.648533215665e-3;  // (eV/Angstrom/amu) -> Angstrom/fs^2
