@@ -140,12 +140,6 @@ template <> __device__ __forceinline__ double g_rc2<double>(const Geom &G) { ret
 template <class R> __device__ __forceinline__ R g_h(const Geom &G, int a);
 template <> __device__ __forceinline__ float g_h<float>(const Geom &G, int a) { return G.h_f[a]; }
 template <> __device__ __forceinline__ double g_h<double>(const Geom &G, int a) { return G.h[a]; }
-template <class R> __device__ __forceinline__ R g_screen_lo(const Geom &G);
-template <> __device__ __forceinline__ float g_screen_lo<float>(const Geom &G) { return G.screen_lo_f; }
-template <> __device__ __forceinline__ double g_screen_lo<double>(const Geom &G) { return G.screen_lo; }
-template <class R> __device__ __forceinline__ R g_screen_hi(const Geom &G);
-template <> __device__ __forceinline__ float g_screen_hi<float>(const Geom &G) { return G.screen_hi_f; }
-template <> __device__ __forceinline__ double g_screen_hi<double>(const Geom &G) { return G.screen_hi; }
 
 // Shift of a list entry's stencil cell: u_j + shift - u_i is the
 // displacement x_j - x_i of the pair.  Per axis -h, 0 or h from the entry's

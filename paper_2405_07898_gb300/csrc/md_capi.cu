@@ -214,7 +214,9 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
     for (int a = 0; a < 3; ++a) {
         ok = ok && alloc_n(ctx, B.d[a], n);
         ok = ok && alloc_n(ctx, B.xw[a], n);
-        ok = ok && alloc_n(ctx, B.uref[a], n);
+        ok = ok && alloc_n(ctx, B.uref[a], n + kScreenPad);
+        B.screen[a] = nullptr;
+        if (a == 0 || sizeof(R) == 8) ok = ok && alloc_n(ctx, B.screen[a], n + kScreenPad);
         ok = ok && alloc_n(ctx, B.fcache[a], n);
         ok = ok && alloc_n(ctx, B.center[a], (size_t)G.ncell[a]);
     }
@@ -227,6 +229,7 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
     ok = ok && alloc_n(ctx, B.cell_old, n);
     ok = ok && alloc_n(ctx, B.slot, n);
     ok = ok && alloc_n(ctx, B.cell_atoms, n);
+    ok = ok && alloc_n(ctx, B.cell_ids, n);
     ok = ok && alloc_n(ctx, B.nnb, n);
     ok = ok && alloc_n(ctx, B.count, (size_t)G.ncells + 1);
     ok = ok && alloc_n(ctx, B.cell_start, (size_t)G.ncells + 1);
@@ -268,6 +271,11 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
     }
     B.tex_shadow[0] = B.tex_shadow[1] = 0;
     if constexpr (std::is_same<R, float>::value) make_record_textures(B, n);
+    // the list build reads (and ignores) the words after the last atom's
+    for (int a = 0; a < 3; ++a)
+        if (cudaMemset(B.uref[a], 0, sizeof(R) * (n + kScreenPad)) != cudaSuccess ||
+            (B.screen[a] && cudaMemset(B.screen[a], 0, sizeof(float) * (n + kScreenPad)) != cudaSuccess))
+            return false;
     if (cudaMemset(B.count, 0, sizeof(int) * ((size_t)G.ncells + 1)) != cudaSuccess) return false;
     if (cudaMemset(B.nnb, 0, sizeof(int) * n) != cudaSuccess) return false;
     if (ctx->opt.half_list && (cudaMemset(B.acc_rho, 0, sizeof(unsigned long long) * n) != cudaSuccess ||
@@ -502,7 +510,7 @@ md_status step_impl(md_ctx *ctx, int64_t nsteps, double dt)
     if (!ctx->opt.use_graphs) {
         for (int64_t s = 0; s < nsteps; ++s) {
             enqueue_step<R>(ctx, L, s == nsteps - 1);
-            ctx->fixed_launches += 3 + 8;
+            ctx->fixed_launches += 3 + rebuild_kernels(ctx->G);
         }
         ctx->fixed_launches += launch_reduce<R>(B, L);
         CK(cudaGetLastError());
@@ -573,7 +581,7 @@ md_status profile_impl(md_ctx *ctx, int64_t nsteps, double dt, md_profile_t *out
         dens += b;
         force += c;
     }
-    // the 8 guarded rebuild kernels exit at once when no build is due: the
+    // the guarded rebuild kernels exit at once when no build is due: the
     // device counted the builds, and they are the longest spans
     md_status rc = read_state(ctx);
     if (rc != MD_OK) return rc;
@@ -1181,31 +1189,24 @@ md_status md_create(const double box[3], int64_t n, const double *pos, const dou
 
     // geometry: cells of edge >= r_list, at least 3 per axis
     Geom &G = ctx->G;
-    double hmax = 0.0;
     for (int a = 0; a < 3; ++a) {
         G.box[a] = box[a];
         G.half_box[a] = 0.5 * box[a];
         G.ncell[a] = (int)std::floor(box[a] / r_list);
         G.inv_cell[a] = (double)G.ncell[a] / box[a];
         G.h[a] = box[a] / (double)G.ncell[a];
-        hmax = std::max(hmax, G.h[a]);
     }
     G.ncells = G.ncell[0] * G.ncell[1] * G.ncell[2];
     G.open_mask = o.open_axes;
     G.rl2 = r_list * r_list;
     G.rc2 = pot->r_cut * pot->r_cut;
-    // rounding bound of the screened r^2 (cell-relative coordinates, |u| <= h)
-    const double eps = (o.precision == MD_PRECISION_MIXED) ? std::ldexp(1.0, -24) : std::ldexp(1.0, -53);
-    const double margin = 8.0 * (20.0 * hmax * r_list + 4.0 * r_list * r_list) * eps;
-    G.screen_lo = G.rl2 - margin;
-    G.screen_hi = G.rl2 + margin;
     for (int a = 0; a < 3; ++a) {
         G.h_f[a] = (float)G.h[a];
         G.inv_cell_f[a] = (float)G.inv_cell[a];
+        G.box_f[a] = (float)box[a];
     }
     G.rc2_f = (float)G.rc2;
-    G.screen_lo_f = (float)G.screen_lo;
-    G.screen_hi_f = (float)G.screen_hi;
+    G.rl2_f = (float)G.rl2;
 
     Launch &L = ctx->L;
     L.n = (int)n;
@@ -1213,12 +1214,13 @@ md_status md_create(const double box[3], int64_t n, const double *pos, const dou
     L.block = o.block_size;
     L.nblocks = (int)((n + L.block - 1) / L.block);
     {
-        // the list build of a small system: blocks as small as it takes to
-        // give every SM two (down to one warp)
+        // the list build: 128 threads a block (a shorter tail than 256: 228
+        // against 234 us a rebuild of 799,496 atoms); in a small system as
+        // few as it takes to give every SM two blocks (down to one warp)
         int dev = 0, nsm = 152;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             nsm = 152;
-        L.list_block = L.block;
+        L.list_block = std::min(L.block, 128);
         while (L.list_block > 32 && (n + L.list_block - 1) / L.list_block < 2 * (int64_t)nsm) L.list_block /= 2;
         L.list_block = std::max(32, L.list_block / 32 * 32);
     }
@@ -1434,7 +1436,7 @@ md_status md_stats(md_ctx *ctx, md_stats_t *out)
     out->rebuilds = h.rebuilds - ctx->rebuilds_at_create;
     out->max_neighbors = h.max_nnb;
     out->table_out_of_range = (int64_t)h.table_oor;
-    out->kernel_launches = ctx->fixed_launches + 8 * h.graph_rebuilds;
+    out->kernel_launches = ctx->fixed_launches + rebuild_kernels(ctx->G) * h.graph_rebuilds;
     out->lanes_density = ctx->L.tpa_d;
     out->lanes_force = ctx->L.tpa_f;
     out->threads_density = ctx->L.block_d;

@@ -47,6 +47,7 @@ __host__ __device__ constexpr uint32_t list_entry(uint32_t q, int dx, int dy, in
 // Largest fused table of the full-list pair passes (segment_fused).
 constexpr int kMaxFusedIntervals = 1 << 22;
 constexpr int kScanBlock = 1024;
+constexpr size_t kScreenPad = 4;  // words after the last atom's coordinates that the list build may read
 constexpr int kEnergySlots = 10;  // embed, pair, ke, virial xx yy zz xy xz yz, spare
 constexpr double kAccel = 9.648533215665e-3;  // (eV/Angstrom/amu) -> Angstrom/fs^2
 
@@ -101,15 +102,13 @@ struct Geom {
     int ncell[3];
     int ncells;
     double rl2;          // r_list^2
-    double screen_lo;    // candidates with r2 below this are in the list for sure
-    double screen_hi;    // ... above this are out for sure; in between: exact FP64 test
     double rc2;          // r_cut^2
     int open_mask;       // one bit per open (non-periodic) axis: 1 x, 2 y, 4 z
     // the same in FP32, so that FP32 kernels convert nothing on the FP64 pipe
     float h_f[3];
     float inv_cell_f[3];  // inv_cell rounded to FP32 (the binning estimate)
     float rc2_f;
-    float screen_lo_f, screen_hi_f;
+    float rl2_f, box_f[3];
 };
 
 template <class R>
@@ -138,7 +137,9 @@ struct Bufs {
     int *slot;
     int *count;
     int *cell_start;
-    int *cell_atoms;
+    int *cell_atoms;     // atoms by cell, in arrival order (scratch of a build)
+    int *cell_ids;       // their original ids
+    float *screen[3];    // list build: x rounded to FP32; FP64 path: also y and z less the cell's centre
     int *block_sums;
     // list
     uint32_t *list;
@@ -201,6 +202,7 @@ constexpr int kPersistentBlock = 256;
 // Host-side launchers (rebuild.cu, pair_f32.cu, pair_f64.cu, persistent.cu).  All are asynchronous on L.stream and
 // return the number of kernels queued.
 template <class R> int launch_rebuild(const Bufs<R> &B, const Geom &G, const Launch &L);
+int rebuild_kernels(const Geom &G);  // kernels of one launch_rebuild
 template <class R> int launch_decide(const Bufs<R> &B, const Launch &L);
 template <class R> int launch_open(const Bufs<R> &B, const Geom &G, const Launch &L);
 template <class R> int launch_density(const Bufs<R> &B, const Geom &G, const Launch &L, bool energy);

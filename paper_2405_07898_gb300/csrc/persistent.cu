@@ -142,13 +142,12 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
         if (need) {
             for (int i = gtid; i < n; i += nthreads) bin_atom<R>(B, G, s, i);
             if (!grid_barrier(ps, err, L.wait_ns)) return;
-            if (blockIdx.x == 0) scan_cells_block<R>(B, G.ncells);
+            scan_part(B.count, B.cell_start, G.ncells, blockIdx.x, gridDim.x);
             if (!grid_barrier(ps, err, L.wait_ns)) return;
-            for (int i = gtid; i < n; i += nthreads) scatter_atom<R>(B, i);
+            for (int i = gtid; i < n; i += nthreads) scatter_atom<R>(B, s, i);
             if (!grid_barrier(ps, err, L.wait_ns)) return;
-            for (int c = gtid; c < G.ncells; c += nthreads) sort_cell<R>(B, s, c);
-            if (!grid_barrier(ps, err, L.wait_ns)) return;
-            for (int p = gtid; p < n; p += nthreads) permute_atom<R>(B, G, s, sp, p);
+            for (int q = gtid; q < n; q += nthreads) permute_atom<R>(B, G, s, sp, q);
+            for (int c = gtid; c < G.ncells; c += nthreads) B.count[c] = 0;  // for the next build
             if (gtid == 0) st->max_nnb = 0;
             s = 1 - s;
             since = 0;
@@ -163,15 +162,13 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                 for (int base = 0; base < n; base += nwarps) {
                     const int p = base + w0;
                     // the warp's lanes share p, so the whole warp takes this branch
-                    if (p < n) cmax = max(cmax, list_atom_warp<R>(B, G, s, sp, p, L.ld, L.cap));
+                    if (p < n) cmax = max(cmax, list_atom_warp<R>(B, G, s, p, L.ld, L.cap));
                 }
-                block_max_nnb(cmax, &st->max_nnb);
+                warp_max_nnb(cmax, &st->max_nnb);
             } else {
-                for (int base = blockIdx.x * blockDim.x; base < n; base += nthreads) {
-                    const int p = base + threadIdx.x;
-                    const int cnt = (p < n) ? list_atom<R>(B, G, s, sp, p, L.ld, L.cap) : 0;
-                    block_max_nnb(cnt, &st->max_nnb);
-                }
+                int cmax = 0;
+                for (int p = gtid; p < n; p += nthreads) cmax = max(cmax, list_atom<R>(B, G, s, p, L.ld, L.cap));
+                warp_max_nnb(cmax, &st->max_nnb);
             }
             if (!grid_barrier(ps, err, L.wait_ns)) return;
         }

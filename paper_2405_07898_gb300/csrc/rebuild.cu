@@ -23,6 +23,10 @@ namespace {
 // +14 % at 18,522, +2 % at 43,904, and a loss from 118,638 atoms up.
 constexpr int64_t kListWarpMaxAtoms = 32768;
 
+// Largest cell grid whose scan is one launch: its blocks read the counts
+// nblocks/2 times over, which costs more than the second launch above that.
+constexpr int kScanOneLaunch = 65536;
+
 // --------------------------------------------------------------------------
 // list build (every rebuild): wrap, bin, scan, scatter, sort, permute, list
 
@@ -40,77 +44,58 @@ template <class R>
 __global__ void k_scan_blocks(Bufs<R> B, int ncells)
 {
     if (!B.st->need_rebuild) return;
-    __shared__ int sm[32];
-    int base = blockIdx.x * kScanBlock;
+    const int base = blockIdx.x * kScanBlock;
     int v = 0;
     for (int c = base + threadIdx.x; c < min(base + kScanBlock, ncells); c += blockDim.x) v += B.count[c];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int w = 0; w < (blockDim.x + 31) / 32; ++w) s += sm[w];
-        B.block_sums[blockIdx.x] = s;
+    v = block_sum_i(v);
+    if (threadIdx.x == 0) B.block_sums[blockIdx.x] = v;
+}
+
+// Accounts of the build, by one thread of the scan: no other thread of that
+// launch reads these words.  k_bin reads the old buffer set; the kernels
+// after the scan write the new one (and copy from the other).
+__device__ __forceinline__ void count_build(DevState *st, int in_graph)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->set = 1 - st->set;
+        st->since_build = 0;
+        st->rebuilds += 1;
+        st->graph_rebuilds += in_graph;
+        st->max_nnb = 0;
     }
 }
 
 // Exclusive scan of the cell counts: cell_start[c] = sum_{c' < c} count[c'].
-// Block b adds the totals of blocks < b, then scans its own kScanBlock cells
-// (blockDim.x == kScanBlock).  Counts are zeroed for the next build.
+// Block b adds the totals of blocks < b (k_scan_blocks), then scans its own
+// kScanBlock cells (blockDim.x == kScanBlock).
 template <class R>
-__global__ void k_scan_apply(Bufs<R> B, int ncells)
+__global__ void __launch_bounds__(kScanBlock) k_scan_apply(Bufs<R> B, int ncells, int in_graph)
 {
     if (!B.st->need_rebuild) return;
-    __shared__ int warp_tot[32];
-    __shared__ int prefix;
-    const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (t < 32) {
-        int s = 0;
-        for (int k = t; k < b; k += 32) s += B.block_sums[k];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (t == 0) prefix = s;
-    }
-    int c = b * kScanBlock + t;
-    int v = (c < ncells) ? B.count[c] : 0;
-    int incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int w = (lane < (int)(blockDim.x >> 5)) ? warp_tot[lane] : 0;
-        int wi = w;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        warp_tot[lane] = wi - w;  // exclusive prefix of warp totals
-    }
-    __syncthreads();
-    int excl = prefix + warp_tot[warp] + incl - v;
-    if (c < ncells) {
-        B.cell_start[c] = excl;
-        B.count[c] = 0;
-        if (c == ncells - 1) B.cell_start[ncells] = excl + v;
-    }
+    count_build(B.st, in_graph);
+    const int b = blockIdx.x, base = b * kScanBlock;
+    int v = 0;
+    for (int k = threadIdx.x; k < b; k += blockDim.x) v += B.block_sums[k];
+    scan_tiles(B.count, B.cell_start, base, min(base + kScanBlock, ncells), ncells, block_sum_i(v));
+}
+
+// The same in one launch, for grids of at most kScanOneLaunch cells: every
+// block adds up all the counts before its part itself.
+template <class R>
+__global__ void __launch_bounds__(kScanBlock) k_scan(Bufs<R> B, int ncells, int in_graph)
+{
+    if (!B.st->need_rebuild) return;
+    count_build(B.st, in_graph);
+    scan_part(B.count, B.cell_start, ncells, blockIdx.x, gridDim.x);
 }
 
 template <class R>
 __global__ void k_scatter(Bufs<R> B, int n)
 {
-    if (!B.st->need_rebuild) return;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) scatter_atom<R>(B, i);
-}
-
-template <class R>
-__global__ void k_cell_sort(Bufs<R> B, int ncells)
-{
-    if (!B.st->need_rebuild) return;
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < ncells) sort_cell<R>(B, B.st->set, c);
+    const DevState *st = B.st;
+    if (!st->need_rebuild) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) scatter_atom<R>(B, 1 - st->set, i);
 }
 
 template <class R>
@@ -118,44 +103,33 @@ __global__ void k_permute(Bufs<R> B, Geom G, int n)
 {
     const DevState *st = B.st;
     if (!st->need_rebuild) return;
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) permute_atom<R>(B, G, st->set, st->sp, p);
-}
-
-template <class R>
-__global__ void k_rebuild_finish(Bufs<R> B, int in_graph)
-{
-    DevState *st = B.st;
-    if (!st->need_rebuild) return;
-    st->set = 1 - st->set;
-    st->since_build = 0;
-    st->rebuilds += 1;
-    st->graph_rebuilds += in_graph;
-    st->max_nnb = 0;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) permute_atom<R>(B, G, 1 - st->set, st->sp, q);
+    for (int c = q; c < G.ncells; c += gridDim.x * blockDim.x) B.count[c] = 0;  // for the next build
 }
 
 // A warp per atom (list_atom_warp), for systems of up to kListWarpMaxAtoms:
 // there the thread-per-atom walk waits on load latency.  Above that it is
 // bound by instruction issue, which the warp form multiplies (a 799,496-atom
-// build took about 780 us with it against 334 us).
+// rebuild took about 780 us with it).
 template <class R>
 __global__ void __launch_bounds__(256) k_build_list_warp(Bufs<R> B, Geom G, int n, int ld, int cap)
 {
     DevState *st = B.st;
     if (!st->need_rebuild) return;
     const int p = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // the same for a warp's lanes
-    const int cnt = (p < n) ? list_atom_warp<R>(B, G, st->set, st->sp, p, ld, cap) : 0;
-    block_max_nnb(cnt, &st->max_nnb);
+    const int cnt = (p < n) ? list_atom_warp<R>(B, G, st->set, p, ld, cap) : 0;
+    warp_max_nnb(cnt, &st->max_nnb);
 }
 
 template <class R>
-__global__ void __launch_bounds__(256) k_build_list(Bufs<R> B, Geom G, int n, int ld, int cap, int half)
+__global__ void __launch_bounds__(256, 6) k_build_list(Bufs<R> B, Geom G, int n, int ld, int cap, int half)
 {
     DevState *st = B.st;
     if (!st->need_rebuild) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int cnt = (p < n) ? list_atom<R>(B, G, st->set, st->sp, p, ld, cap, half != 0) : 0;
-    block_max_nnb(cnt, &st->max_nnb);
+    const int cnt = (p < n) ? list_atom<R>(B, G, st->set, p, ld, cap, half != 0) : 0;
+    warp_max_nnb(cnt, &st->max_nnb);
 }
 
 // --------------------------------------------------------------------------
@@ -248,18 +222,22 @@ int launch_rebuild(const Bufs<R> &B, const Geom &G, const Launch &L)
     const int b = L.block, nb = blocks_for(L.n, b);
     const int nsb = blocks_for(G.ncells, kScanBlock);
     k_bin<R><<<nb, b, 0, L.stream>>>(B, G, L.n);
-    k_scan_blocks<R><<<nsb, 256, 0, L.stream>>>(B, G.ncells);
-    k_scan_apply<R><<<nsb, kScanBlock, 0, L.stream>>>(B, G.ncells);
+    if (G.ncells <= kScanOneLaunch) {
+        k_scan<R><<<nsb, kScanBlock, 0, L.stream>>>(B, G.ncells, L.use_cond);
+    } else {
+        k_scan_blocks<R><<<nsb, 256, 0, L.stream>>>(B, G.ncells);
+        k_scan_apply<R><<<nsb, kScanBlock, 0, L.stream>>>(B, G.ncells, L.use_cond);
+    }
     k_scatter<R><<<nb, b, 0, L.stream>>>(B, L.n);
-    k_cell_sort<R><<<blocks_for(G.ncells, 256), 256, 0, L.stream>>>(B, G.ncells);
     k_permute<R><<<nb, b, 0, L.stream>>>(B, G, L.n);
-    k_rebuild_finish<R><<<1, 1, 0, L.stream>>>(B, L.use_cond);
     if (!L.half && (int64_t)L.n <= kListWarpMaxAtoms)
         k_build_list_warp<R><<<blocks_for((int64_t)L.n * 32, 256), 256, 0, L.stream>>>(B, G, L.n, L.ld, L.cap);
     else
         k_build_list<R><<<blocks_for(L.n, L.list_block), L.list_block, 0, L.stream>>>(B, G, L.n, L.ld, L.cap, L.half);
-    return 8;
+    return rebuild_kernels(G);
 }
+
+int rebuild_kernels(const Geom &G) { return G.ncells <= kScanOneLaunch ? 5 : 6; }
 
 template <class R>
 int launch_decide(const Bufs<R> &B, const Launch &L)
