@@ -100,7 +100,7 @@ struct md_ctx {
     double *adj_host = nullptr;   // pinned: |g|^2, then the knot gradient
     // persistent step launch (md_step as one cooperative kernel)
     PersistScratch *ps = nullptr;
-    int persist_tpa = 0, persist_grid = 0;  // 0: graph path
+    PersistSched persist{};  // grid 0: graph path
     std::string err;
 
     md_status fail(md_status s, const std::string &m)
@@ -501,8 +501,8 @@ md_status step_impl(md_ctx *ctx, int64_t nsteps, double dt)
     Launch L = ctx->L;
     L.use_cond = 0;
     L.cond = 0;
-    if (ctx->persist_grid > 0) {
-        CK(launch_steps<R>(B, ctx->G, L, nsteps, ctx->persist_tpa, ctx->persist_grid, ctx->ps));
+    if (ctx->persist.grid > 0) {
+        CK(launch_steps<R>(B, ctx->G, L, nsteps, ctx->persist, ctx->ps));
         ctx->fixed_launches += 1;
         return MD_OK;
     }
@@ -738,11 +738,16 @@ md_status autotune(md_ctx *ctx)
     const Bufs<R> &B = bufs<R>(ctx);
     // block sizes below 256 let the atom-parallel passes fill their last
     // wave of blocks on the GPU
+    int dev = 0, nsm = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     std::vector<PassSched> cand;
     for (int t : {1, 2})
         for (int b : {128, 256, 192, 224, 160, 96, 64}) cand.push_back({t, b});
-    cand.push_back({4, 256});
-    cand.push_back({8, 256});
+    // many lanes: smaller blocks where 256 threads leave SMs without work
+    for (int t : {4, 8})
+        for (int b : {256, 128, 64})
+            if (b == 256 || blocks_for_host((int64_t)ctx->n * t, 2 * b) < 2 * nsm) cand.push_back({t, b});
     const int nc = (int)cand.size();
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
@@ -818,7 +823,7 @@ constexpr int64_t kPersistentAutoAtoms = 65536;
 template <class R>
 md_status setup_persistent(md_ctx *ctx)
 {
-    ctx->persist_grid = 0;
+    ctx->persist = PersistSched{};
     const md_options &o = ctx->opt;
     const bool want = o.persistent == MD_PERSIST_ON || (o.persistent == MD_PERSIST_AUTO && ctx->n <= kPersistentAutoAtoms);
     if (!want || ctx->n == 0) return MD_OK;
@@ -835,25 +840,28 @@ md_status setup_persistent(md_ctx *ctx)
     if (o.lanes_per_atom > 0) tpas.push_back(o.lanes_per_atom);
     else if (ctx->L.rebuild_every < 2) tpas.push_back(2);  // every step builds: no state-neutral trial
     else tpas = {1, 2, 4, 8};
-    struct Cand {
-        int tpa, grid;
-    };
-    std::vector<Cand> cand;
-    for (int tpa : tpas) {
-        if (!coop) break;
-        const int grid = persistent_grid<R>(ctx->L, tpa);
-        if (grid > 0) cand.push_back({tpa, grid});
-    }
+    // blocks of 256 threads, and smaller ones where those leave SMs without
+    // work: a small system's phases are chains of latencies and, in FP64, of
+    // the SM's narrow FP64 pipe, so every SM should have its share (2,000
+    // atoms in FP64, 8 lanes each: 27.8 us a step in 63 blocks of 256 threads,
+    // 20.1 in 125 of 128).  Larger blocks need fewer arrivals at the barriers
+    // (43,904 atoms: 23.7 us in 343 blocks, 24.3 in 686, 2 lanes each).
+    int nsm = 0;
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    std::vector<PersistSched> cand;
+    for (int tpa : tpas)
+        for (int block : {256, 128, 64}) {
+            if (!coop) break;
+            const int grid = persistent_grid<R>(ctx->L, tpa, block);
+            if (grid > 0) cand.push_back({tpa, block, grid});
+            if (grid >= 2 * nsm) break;
+        }
     if (cand.empty()) {
         if (forced) return ctx->fail(MD_ERR_CUDA, "the persistent step kernel cannot be resident");
         return MD_OK;
     }
-    auto take = [&](const Cand &c) {
-        ctx->persist_tpa = c.tpa;
-        ctx->persist_grid = c.grid;
-    };
     if (cand.size() == 1 || ctx->L.rebuild_every < 2) {
-        take(cand[0]);
+        ctx->persist = cand[0];
         return MD_OK;
     }
     const int trial_steps = ctx->L.rebuild_every - 1;
@@ -870,9 +878,8 @@ md_status setup_persistent(md_ctx *ctx)
     int best_i = -1;
     for (int round = 0; round < 3; ++round) {
         for (size_t c = 0; c < cand.size(); ++c) {
-            const Cand &k = cand[c];
             CK(cudaEventRecord(e0, ctx->stream));
-            CK(launch_steps<R>(B, ctx->G, L, trial_steps, k.tpa, k.grid, ctx->ps));
+            CK(launch_steps<R>(B, ctx->G, L, trial_steps, cand[c], ctx->ps));
             CK(cudaEventRecord(e1, ctx->stream));
             CK(cudaEventSynchronize(e1));
             float ms = 0.f;
@@ -889,7 +896,7 @@ md_status setup_persistent(md_ctx *ctx)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (saved.error) return check_device_errors(ctx);
-    take(cand[best_i]);
+    ctx->persist = cand[best_i];
     return check_device_errors(ctx);
 }
 
@@ -1224,7 +1231,7 @@ md_status md_create(const double box[3], int64_t n, const double *pos, const dou
         while (L.list_block > 32 && (n + L.list_block - 1) / L.list_block < 2 * (int64_t)nsm) L.list_block /= 2;
         L.list_block = std::max(32, L.list_block / 32 * 32);
     }
-    L.pstride = std::max(1, blocks_for_host(8 * n, std::min(L.block, 128)));
+    L.pstride = std::max(1, blocks_for_host(8 * n, std::min(L.block, 64)));
     {
         int lanes = o.lanes_per_atom > 0 ? o.lanes_per_atom : (o.half_list ? 1 : 4);
         L.tpa_d = L.tpa_f = lanes;
@@ -1441,8 +1448,8 @@ md_status md_stats(md_ctx *ctx, md_stats_t *out)
     out->lanes_force = ctx->L.tpa_f;
     out->threads_density = ctx->L.block_d;
     out->threads_force = ctx->L.block_f;
-    out->persistent_blocks = ctx->persist_grid;
-    out->persistent_lanes = ctx->persist_grid ? ctx->persist_tpa : 0;
+    out->persistent_blocks = ctx->persist.grid;
+    out->persistent_lanes = ctx->persist.grid ? ctx->persist.tpa : 0;
     out->half_list = ctx->L.half;
     out->record_textures = (ctx->precision == MD_PRECISION_MIXED && ctx->Bf.tex_shadow[0] && ctx->Bf.tex_shadow[1]) ? 1 : 0;
     return MD_OK;

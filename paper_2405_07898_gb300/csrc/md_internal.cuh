@@ -197,7 +197,11 @@ struct PersistScratch {
     unsigned long long arrive;
     unsigned maxdisp[2];
 };
-constexpr int kPersistentBlock = 256;
+// Shape of the persistent launch: lanes per atom, threads per block, blocks
+// (0: not launched).
+struct PersistSched {
+    int tpa, block, grid;
+};
 
 // Host-side launchers (rebuild.cu, pair_f32.cu, pair_f64.cu, persistent.cu).  All are asynchronous on L.stream and
 // return the number of kernels queued.
@@ -207,12 +211,13 @@ template <class R> int launch_decide(const Bufs<R> &B, const Launch &L);
 template <class R> int launch_open(const Bufs<R> &B, const Geom &G, const Launch &L);
 template <class R> int launch_density(const Bufs<R> &B, const Geom &G, const Launch &L, bool energy);
 template <class R> int launch_force(const Bufs<R> &B, const Geom &G, const Launch &L, int mode, bool energy);
-// md_step as one cooperative launch of `grid` blocks with `tpa` lanes per atom
-// in the pair passes (persistent.cu); persistent_grid: the blocks that can be
-// resident at once for that kernel (0 if it cannot be launched).
-template <class R> int persistent_grid(const Launch &L, int tpa);
+// md_step as one cooperative launch (persistent.cu); persistent_grid: the
+// blocks of `block` threads (a multiple of 32, at most 256) with `tpa` lanes
+// per atom that n atoms need and that can be resident at once (0 if the
+// kernel cannot be launched).
+template <class R> int persistent_grid(const Launch &L, int tpa, int block);
 template <class R>
-cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, int tpa, int grid,
+cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, const PersistSched &sched,
                          PersistScratch *ps);
 
 template <class R> int launch_reduce(const Bufs<R> &B, const Launch &L);

@@ -172,14 +172,23 @@ __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R r
     const SplineDesc<R> g = MULTI ? T.f[0] : T.fphi;
     const Own<R> own(ui, h);
     R rho = (R)0;
-    (void)cap;
+    // Many lanes per atom (small systems, bound by latency): the columns of
+    // the first round are read before the neighbour count is known, as in the
+    // force pass.  With few lanes the registers cost more than the wait.
+    constexpr bool kEarly = TPA >= 4;
+    uint32_t e[U];
+    if (kEarly) {
+#pragma unroll
+        for (int q = 0; q < U; ++q) e[q] = (l + q * TPA < cap) ? list(l + q * TPA) : 0u;
+    }
     const int nn = *nnb_i;
     // U pairs per round (columns k, k + TPA, ...), all gathers issued before
     // any is used; the sum runs in column order
     for (int k = l; k < nn; k += U * TPA) {
-        uint32_t e[U];
+        if (!kEarly || k != l) {
 #pragma unroll
-        for (int q = 0; q < U; ++q) e[q] = (k + q * TPA < nn) ? list(k + q * TPA) : 0u;
+            for (int q = 0; q < U; ++q) e[q] = (k + q * TPA < nn) ? list(k + q * TPA) : 0u;
+        }
         R4 u[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) u[q] = fetch(q == 0 || k + q * TPA < nn ? e[q] : e[0]);

@@ -277,24 +277,24 @@ const void *steps_kernel(int tpa)
 }  // namespace
 
 template <class R>
-int persistent_grid(const Launch &L, int tpa)
+int persistent_grid(const Launch &L, int tpa, int block)
 {
     const void *fn = L.multi ? steps_kernel<R, true>(tpa) : steps_kernel<R, false>(tpa);
     int per_sm = 0, dev = 0, nsm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPersistentBlock, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, 0) != cudaSuccess ||
         cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm <= 0)
         return 0;
-    const int width = kPersistentBlock / tpa;
+    const int width = block / tpa;
     const int ntiles = (L.n + width - 1) / width;
     return std::max(1, std::min(ntiles, per_sm * nsm));
 }
 
 template <class R>
-cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, int tpa, int grid,
+cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, const PersistSched &sched,
                          PersistScratch *ps)
 {
-    const void *fn = L.multi ? steps_kernel<R, true>(tpa) : steps_kernel<R, false>(tpa);
+    const void *fn = L.multi ? steps_kernel<R, true>(sched.tpa) : steps_kernel<R, false>(sched.tpa);
     Bufs<R> b = B;
     Geom g = G;
     Launch l = L;
@@ -303,14 +303,14 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
     void *args[] = {&b, &g, &l, &ns, &p};
     cudaError_t e = cudaMemsetAsync(&ps->arrive, 0, sizeof(ps->arrive), L.stream);
     if (e != cudaSuccess) return e;
-    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kPersistentBlock), args, 0, L.stream);
+    return cudaLaunchCooperativeKernel(fn, dim3(sched.grid), dim3(sched.block), args, 0, L.stream);
 }
 
-template int persistent_grid<float>(const Launch &, int);
-template int persistent_grid<double>(const Launch &, int);
-template cudaError_t launch_steps<float>(const Bufs<float> &, const Geom &, const Launch &, long long, int, int,
-                                         PersistScratch *);
-template cudaError_t launch_steps<double>(const Bufs<double> &, const Geom &, const Launch &, long long, int, int,
-                                          PersistScratch *);
+template int persistent_grid<float>(const Launch &, int, int);
+template int persistent_grid<double>(const Launch &, int, int);
+template cudaError_t launch_steps<float>(const Bufs<float> &, const Geom &, const Launch &, long long,
+                                         const PersistSched &, PersistScratch *);
+template cudaError_t launch_steps<double>(const Bufs<double> &, const Geom &, const Launch &, long long,
+                                          const PersistSched &, PersistScratch *);
 
 }  // namespace eammd
