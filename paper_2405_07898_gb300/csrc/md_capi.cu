@@ -816,6 +816,20 @@ md_status autotune(md_ctx *ctx)
 // graph replay (measured on GB300 over the BCC sweep).
 constexpr int64_t kPersistentAutoAtoms = 65536;
 
+// Shapes of the persistent launch that were timed, per (device, precision, type
+// path, list capacity, quarter octave of the size), kept for the life of the
+// process as the pair passes' schedules are: contexts of the same shape run
+// the same lanes per atom, and only the first pays for the trials.
+struct PersistKey {
+    int dev, precision, multi, cap, bucket;
+    bool operator==(const PersistKey &o) const
+    {
+        return dev == o.dev && precision == o.precision && multi == o.multi && cap == o.cap && bucket == o.bucket;
+    }
+};
+std::vector<std::pair<PersistKey, PersistSched>> g_persist_cache;  // under g_tune_mu
+constexpr size_t kPersistCacheMax = 256;
+
 // The persistent step launch: a cooperative grid of as many blocks as are
 // resident.  Lanes per atom come from the options, else every feasible
 // choice is timed over rebuild_every - 1 steps at dt = 0, which moves no atom
@@ -840,6 +854,20 @@ md_status setup_persistent(md_ctx *ctx)
     if (o.lanes_per_atom > 0) tpas.push_back(o.lanes_per_atom);
     else if (ctx->L.rebuild_every < 2) tpas.push_back(2);  // every step builds: no state-neutral trial
     else tpas = {1, 2, 4, 8};
+    const PersistKey key{dev, ctx->precision, ctx->L.multi, ctx->L.cap, (int)(4.0 * std::log2((double)ctx->n))};
+    const bool timed = o.lanes_per_atom == 0 && ctx->L.rebuild_every >= 2;
+    if (timed && coop) {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        for (auto &e : g_persist_cache)
+            if (e.first == key) {
+                PersistSched k = e.second;
+                k.grid = persistent_grid<R>(ctx->L, k.tpa, k.block);
+                if (k.grid > 0) {
+                    ctx->persist = k;
+                    return MD_OK;
+                }
+            }
+    }
     // blocks of 256 threads, and smaller ones where those leave SMs without
     // work: a small system's phases are chains of latencies and, in FP64, of
     // the SM's narrow FP64 pipe, so every SM should have its share (2,000
@@ -897,6 +925,10 @@ md_status setup_persistent(md_ctx *ctx)
     cudaEventDestroy(e1);
     if (saved.error) return check_device_errors(ctx);
     ctx->persist = cand[best_i];
+    if (timed) {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        if (g_persist_cache.size() < kPersistCacheMax) g_persist_cache.push_back({key, ctx->persist});
+    }
     return check_device_errors(ctx);
 }
 

@@ -33,13 +33,6 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
     return v;
 }
 
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(__cvta_generic_to_global(p)) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long *p)
 {
     unsigned long long v;
@@ -48,39 +41,35 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
 }
 
 // Grid barrier on a counter that only grows during a launch (zeroed by the
-// host before it): barrier b of the launch is passed once the counter reaches
-// (b + 1) x gridDim.x.  Arrival is a release add, the wait an acquire load, so
-// every block sees the writes all blocks made before the barrier.  Returns
-// false once any wait of the launch has timed out.
-__device__ __forceinline__ bool grid_barrier(PersistScratch *ps, unsigned *err, uint64_t wait_ns)
+// host before it): barrier b of the launch (b = 1, 2, ...) is passed once the
+// counter reaches b x gridDim.x.  Arrival is a release add whose result
+// nobody waits for (every block counts the barriers itself); the wait polls
+// with acquire loads, so every block sees the writes all blocks made before
+// the barrier.  A trip to L2 is about 0.4 us and a barrier is a chain of them:
+// the fence of the release, the add, the polls.  (1,024 atoms, 2.6 barriers a
+// step: 11.35 us a step with the add's result waited for, the error word read
+// first and relaxed polls before one acquire load, 11.26 with relaxed polls
+// and a fence, 10.45 so.)
+// Returns false once a wait of the launch has timed out (a block that waits
+// looks at the error word every 64th poll; one that gave up arrives no more,
+// so nobody passes a later barrier).
+__device__ __forceinline__ bool grid_barrier(PersistScratch *ps, unsigned *err, uint64_t wait_ns,
+                                             unsigned long long &target)
 {
     __shared__ int ok;
+    target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
         int good = 1;
-        if (ld_acquire(err) & ERR_TIMEOUT) {
-            good = 0;
-        } else {
-            unsigned long long a;
-            asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;"
-                         : "=l"(a)
-                         : "l"(__cvta_generic_to_global(&ps->arrive))
-                         : "memory");
-            const unsigned long long g = gridDim.x;
-            const unsigned long long target = (a / g + 1) * g;
-            if (a + 1 != target) {
-                // relaxed polls, one acquire load once the count is reached;
-                // the error word and the clock are read every 64th poll only
-                const uint64_t t0 = global_ns();
-                unsigned spins = 0;
-                while (ld_relaxed(&ps->arrive) < target || ld_acquire(&ps->arrive) < target) {
-                    if ((++spins & 63u) == 0 &&
-                        ((ld_acquire(err) & ERR_TIMEOUT) || global_ns() - t0 > wait_ns)) {
-                        atomicOr(err, ERR_TIMEOUT);
-                        good = 0;
-                        break;
-                    }
-                    __nanosleep(16);
+        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(__cvta_generic_to_global(&ps->arrive)) : "memory");
+        if (ld_acquire(&ps->arrive) < target) {
+            const uint64_t t0 = global_ns();
+            unsigned spins = 0;
+            while (ld_acquire(&ps->arrive) < target) {
+                if ((++spins & 63u) == 0 && ((ld_acquire(err) & ERR_TIMEOUT) || global_ns() - t0 > wait_ns)) {
+                    atomicOr(err, ERR_TIMEOUT);
+                    good = 0;
+                    break;
                 }
             }
         }
@@ -110,6 +99,10 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
     constexpr int UD = PairsInFlight<MULTI>::density, UF = PairsInFlight<MULTI>::force;
     DevState *st = B.st;
     unsigned *err = &st->error;
+    unsigned long long target = 0;  // of the grid barriers
+    // a launch that timed out left its phase half done: nothing runs on it
+    // until the state is set anew (the error word is cleared then)
+    if (__syncthreads_or((int)(ld_acquire(err) & ERR_TIMEOUT))) return;
     int s = st->set, sp = st->sp, since = st->since_build;
     long long step = st->step, rebuilds = 0;
     int need = 0;
@@ -126,7 +119,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
         for (int i = gtid; i < n; i += nthreads) d2 = fmaxf(d2, open_atom<R>(B, L, s, sp, i));
         block_max_disp(d2, &ps->maxdisp[1]);
     }
-    if (!grid_barrier(ps, err, L.wait_ns)) return;
+    if (!grid_barrier(ps, err, L.wait_ns, target)) return;
 
     for (long long k = 0; k < nsteps; ++k) {
         const bool last = k == nsteps - 1;
@@ -141,18 +134,18 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
 
         if (need) {
             for (int i = gtid; i < n; i += nthreads) bin_atom<R>(B, G, s, i);
-            if (!grid_barrier(ps, err, L.wait_ns)) return;
+            if (!grid_barrier(ps, err, L.wait_ns, target)) return;
             scan_part(B.count, B.cell_start, G.ncells, blockIdx.x, gridDim.x);
-            if (!grid_barrier(ps, err, L.wait_ns)) return;
+            if (!grid_barrier(ps, err, L.wait_ns, target)) return;
             for (int i = gtid; i < n; i += nthreads) scatter_atom<R>(B, s, i);
-            if (!grid_barrier(ps, err, L.wait_ns)) return;
+            if (!grid_barrier(ps, err, L.wait_ns, target)) return;
             for (int q = gtid; q < n; q += nthreads) permute_atom<R>(B, G, s, sp, q);
             for (int c = gtid; c < G.ncells; c += nthreads) B.count[c] = 0;  // for the next build
             if (gtid == 0) st->max_nnb = 0;
             s = 1 - s;
             since = 0;
             rebuilds += 1;
-            if (!grid_barrier(ps, err, L.wait_ns)) return;
+            if (!grid_barrier(ps, err, L.wait_ns, target)) return;
             if ((long long)n * 32 <= (long long)nthreads * kListWarpPasses) {
                 // a warp per atom, one lane per stencil cell; the grid's warps
                 // take the atoms in at most kListWarpPasses passes
@@ -170,7 +163,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                 for (int p = gtid; p < n; p += nthreads) cmax = max(cmax, list_atom<R>(B, G, s, p, L.ld, L.cap));
                 warp_max_nnb(cmax, &st->max_nnb);
             }
-            if (!grid_barrier(ps, err, L.wait_ns)) return;
+            if (!grid_barrier(ps, err, L.wait_ns, target)) return;
         }
 
         // density pass
@@ -193,7 +186,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                 block_sums_t<1, R>(v, B.partials, L.pstride, 0);
             }
         }
-        if (!grid_barrier(ps, err, L.wait_ns)) return;
+        if (!grid_barrier(ps, err, L.wait_ns, target)) return;
 
         // force pass with the closing kick (and, but for the last step, the
         // next opening kick and the drift)
@@ -245,7 +238,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                 block_max_disp(d2max, &ps->maxdisp[k & 1]);
             }
         }
-        if (!grid_barrier(ps, err, L.wait_ns)) return;
+        if (!grid_barrier(ps, err, L.wait_ns, target)) return;
     }
 
     // energies of the last step, counters back to DevState
