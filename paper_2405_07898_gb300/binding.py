@@ -336,13 +336,13 @@ class MD:
         return w
 
     def forces(self, out=None):
-        out = np.zeros((self.n, 3)) if out is None else out
+        out = np.empty((self.n, 3)) if out is None else out
         self._check(self._L.md_forces(self.h, _d(out) if isinstance(out, np.ndarray) else _ptr(out)))
         return out
 
     def get_state(self, pos=None, vel=None):
-        pos = np.zeros((self.n, 3)) if pos is None else pos
-        vel = np.zeros((self.n, 3)) if vel is None else vel
+        pos = np.empty((self.n, 3)) if pos is None else pos
+        vel = np.empty((self.n, 3)) if vel is None else vel
         st = C.c_int64()
         self._check(self._L.md_get_state(self.h, _ptr(pos), _ptr(vel), C.byref(st)))
         return pos, vel, st.value
@@ -479,7 +479,7 @@ class MDBatch:
 
     def get_state(self, r: int):
         n = self.systems[r].n
-        pos, vel, force = np.zeros((n, 3)), np.zeros((n, 3)), np.zeros((n, 3))
+        pos, vel, force = np.empty((n, 3)), np.empty((n, 3)), np.empty((n, 3))
         self._check(self._L.md_batch_get_state(self.h, int(r), _ptr(pos), _ptr(vel), _ptr(force)))
         return pos, vel, force
 

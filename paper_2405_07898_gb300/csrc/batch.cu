@@ -645,7 +645,11 @@ struct md_batch {
     std::vector<RepParam> par;
     std::vector<int> order;
     BatchBufs B{};
-    RepState *st_host = nullptr;
+    RepState *st_host = nullptr;    // pinned
+    bool st_current = false;        // st_host holds the device's states, st_status what they say
+    md_status st_status = MD_OK;
+    std::string st_message;
+    double *host_stage = nullptr;   // pinned: positions, velocities, forces of one replica
     std::vector<void *> allocs;
     md_options opt{};
     cudaStream_t stream = nullptr;
@@ -705,6 +709,7 @@ constexpr int kNumSchedules = 5;
 
 md_status batch_launch(md_batch *b, int mode, int nsteps, double dt)
 {
+    b->st_current = false;
     BCK(cudaMemsetAsync(b->B.queue, 0, sizeof(int), b->stream));
     switch (b->schedule) {
     case 1: k_batch<256, 2><<<b->grid, 256, 0, b->stream>>>(b->B, mode, nsteps, dt); break;
@@ -718,19 +723,34 @@ md_status batch_launch(md_batch *b, int mode, int nsteps, double dt)
     return MD_OK;
 }
 
+// Waits for the stream; after new work also reads every replica's state and
+// finds the first error.  With nothing queued since, the states and the
+// answer read last still stand.
 md_status batch_sync(md_batch *b)
 {
+    if (!b->st_current)
+        BCK(cudaMemcpyAsync(b->st_host, b->B.st, sizeof(RepState) * b->nrep, cudaMemcpyDeviceToHost, b->stream));
     BCK(cudaStreamSynchronize(b->stream));
-    BCK(cudaMemcpy(b->st_host, b->B.st, sizeof(RepState) * b->nrep, cudaMemcpyDeviceToHost));
-    for (int r = 0; r < b->nrep; ++r) {
-        const unsigned e = b->st_host[r].error;
-        if (e & ERR_LIST_OVERFLOW)
-            return b->fail(MD_ERR_LIST_OVERFLOW, "replica " + std::to_string(r) + ": list capacity exceeded (" +
-                                                     std::to_string(b->st_host[r].max_nnb) + " > " +
-                                                     std::to_string(b->B.cap) + ")");
-        if (e & ERR_NONFINITE) return b->fail(MD_ERR_NONFINITE, "replica " + std::to_string(r) + ": non-finite force");
+    if (!b->st_current) {
+        b->st_current = true;
+        b->st_status = MD_OK;
+        b->st_message.clear();
+        for (int r = 0; r < b->nrep; ++r) {
+            const unsigned e = b->st_host[r].error;
+            if (e & ERR_LIST_OVERFLOW) {
+                b->st_status = MD_ERR_LIST_OVERFLOW;
+                b->st_message = "replica " + std::to_string(r) + ": list capacity exceeded (" +
+                                std::to_string(b->st_host[r].max_nnb) + " > " + std::to_string(b->B.cap) + ")";
+                break;
+            }
+            if (e & ERR_NONFINITE) {
+                b->st_status = MD_ERR_NONFINITE;
+                b->st_message = "replica " + std::to_string(r) + ": non-finite force";
+                break;
+            }
+        }
     }
-    return MD_OK;
+    return b->st_status == MD_OK ? MD_OK : b->fail(b->st_status, b->st_message);
 }
 
 }  // namespace
@@ -910,6 +930,7 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
     if (ce == cudaSuccess) ce = cudaMemset(B.count, 0, sizeof(int) * (size_t)cell_off);
     if (ce == cudaSuccess) ce = cudaMemset(B.st, 0, sizeof(RepState) * (size_t)nrep);
     if (ce == cudaSuccess) ce = cudaMallocHost((void **)&b->st_host, sizeof(RepState) * nrep);
+    if (ce == cudaSuccess) ce = cudaMallocHost((void **)&b->host_stage, sizeof(double) * 9 * (size_t)b->max_n);
     // per-replica state, caller order within each replica
     for (int r = 0; r < nrep && ce == cudaSuccess; ++r) {
         const md_replica &R = reps[r];
@@ -985,6 +1006,7 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
                     best = ms;
                     best_s = sc;
                 }
+                b->st_current = false;  // the device state is restored below
                 if (rc == MD_OK && cudaMemcpy(B.st, b->st_host, sizeof(RepState) * nrep, cudaMemcpyHostToDevice) != cudaSuccess)
                     rc = MD_ERR_CUDA;
                 if (rc == MD_OK) {
@@ -1014,6 +1036,7 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
     }
     // rebuild counters start after the initial build
     for (int r = 0; r < nrep; ++r) b->st_host[r].rebuilds = 0;
+    b->st_current = false;
     if (cudaMemcpy(B.st, b->st_host, sizeof(RepState) * nrep, cudaMemcpyHostToDevice) != cudaSuccess) {
         md_batch_destroy(b);
         return bad(MD_ERR_CUDA, "state upload failed");
@@ -1030,6 +1053,7 @@ md_status md_batch_step(md_batch *b, int64_t nsteps, double dt)
     if (!b->opt.use_graphs) return batch_launch(b, BATCH_RUN, (int)nsteps, dt);
     for (auto &g : b->graphs)
         if (g.nsteps == (int)nsteps && g.dt == dt) {
+            b->st_current = false;
             BCK(cudaGraphLaunch(g.e, b->stream));
             b->launches += 1;
             return MD_OK;
@@ -1049,6 +1073,7 @@ md_status md_batch_step(md_batch *b, int64_t nsteps, double dt)
     cudaGraphExec_t ex;
     BCK(cudaGraphInstantiate(&ex, g, 0));
     b->graphs.push_back({(int)nsteps, dt, g, ex});
+    b->st_current = false;
     BCK(cudaGraphLaunch(ex, b->stream));
     b->launches += 1;
     return MD_OK;
@@ -1072,16 +1097,25 @@ md_status md_batch_get_state(md_batch *b, int32_t r, double *pos, double *vel, d
     if (r < 0 || r >= b->nrep) return b->fail(MD_ERR_ARG, "replica index out of range");
     md_status rc = batch_sync(b);
     if (rc != MD_OK) return rc;
-    const int n = b->par[r].n;
-    double *dp = b->stage, *dv = b->stage + 3 * (size_t)n, *df = b->stage + 6 * (size_t)n;
-    k_batch_store<<<(n + 255) / 256, 256, 0, b->stream>>>(b->B, r, pos ? dp : nullptr, vel ? dv : nullptr,
-                                                          force ? df : nullptr);
+    const size_t n = (size_t)b->par[r].n;
+    // gathered on the device, one copy to pinned memory, then into the
+    // caller's arrays (a copy per array into pageable memory took 230 us a
+    // replica of 5,900 atoms)
+    double *out[3] = {pos, vel, force}, *at[3] = {nullptr, nullptr, nullptr};
+    size_t len = 0;
+    for (int k = 0; k < 3; ++k)
+        if (out[k]) {
+            at[k] = b->stage + len;
+            len += 3 * n;
+        }
+    if (len == 0) return MD_OK;
+    k_batch_store<<<(int)((n + 255) / 256), 256, 0, b->stream>>>(b->B, r, at[0], at[1], at[2]);
     b->launches += 1;
     BCK(cudaGetLastError());
-    if (pos) BCK(cudaMemcpyAsync(pos, dp, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, b->stream));
-    if (vel) BCK(cudaMemcpyAsync(vel, dv, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, b->stream));
-    if (force) BCK(cudaMemcpyAsync(force, df, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, b->stream));
+    BCK(cudaMemcpyAsync(b->host_stage, b->stage, sizeof(double) * len, cudaMemcpyDeviceToHost, b->stream));
     BCK(cudaStreamSynchronize(b->stream));
+    for (int k = 0; k < 3; ++k)
+        if (out[k]) memcpy(out[k], b->host_stage + (at[k] - b->stage), sizeof(double) * 3 * n);
     return MD_OK;
 }
 
@@ -1120,6 +1154,7 @@ void md_batch_destroy(md_batch *b)
         else cudaFree(p);
     }
     if (b->st_host) cudaFreeHost(b->st_host);
+    if (b->host_stage) cudaFreeHost(b->host_stage);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
 }

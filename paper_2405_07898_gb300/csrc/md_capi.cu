@@ -55,6 +55,9 @@ bool spline_ok(const md_spline &s)
     return true;
 }
 
+// Largest system whose state is stored straight into pinned host memory.
+constexpr int64_t kHostStageAtoms = 8192;
+
 struct GraphEntry {
     int kind;     // 0 = middle steps, 1 = closing step
     int nsteps;
@@ -82,6 +85,8 @@ struct md_ctx {
     Bufs<double> Bd{};
     DevState *st = nullptr;
     DevState *st_host = nullptr;  // pinned
+    bool st_current = false;      // st_host is the device state (read_state, touch)
+    double *host_stage = nullptr; // pinned, kHostStageAtoms or fewer: AoS pos, vel, force
     double *stage = nullptr;      // 9 n doubles: AoS pos, vel, force
     int *types_orig = nullptr;
     std::vector<GraphEntry> graphs;
@@ -308,12 +313,21 @@ bool grow_list(md_ctx *ctx, int cap)
     return true;
 }
 
+// The device state into st_host, after the work queued so far: the copy goes
+// behind it on the stream and one wait ends both.  st_host stays current until
+// something that changes the device state is queued (touch); later calls then
+// only wait for the stream.
 md_status read_state(md_ctx *ctx)
 {
+    if (!ctx->st_current)
+        CK(cudaMemcpyAsync(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaMemcpy(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost));
+    ctx->st_current = true;
     return MD_OK;
 }
+
+// To be called wherever kernels or copies that write the device state are queued.
+void touch(md_ctx *ctx) { ctx->st_current = false; }
 
 // The error flags of the device state last read into st_host.
 md_status state_errors(md_ctx *ctx)
@@ -340,6 +354,7 @@ md_status check_device_errors(md_ctx *ctx)
 template <class R>
 md_status measure(md_ctx *ctx)
 {
+    touch(ctx);
     const Bufs<R> &B = bufs<R>(ctx);
     Launch L = ctx->L;
     L.use_cond = 0;
@@ -359,6 +374,7 @@ md_status load_and_measure(md_ctx *ctx, const double *pos, const double *vel, in
 {
     const Bufs<R> &B0 = bufs<R>(ctx);
     const size_t n = (size_t)ctx->n;
+    touch(ctx);
     // the permutation restarts from the caller's order in buffer set 0
     DevState h{};
     h.step = step;
@@ -495,6 +511,7 @@ template <class R> md_status setup_persistent(md_ctx *ctx);
 template <class R>
 md_status step_impl(md_ctx *ctx, int64_t nsteps, double dt)
 {
+    touch(ctx);
     const Bufs<R> &B = bufs<R>(ctx);
     ctx->L.dt = dt;
     for (int t = 0; t < ctx->ntypes; ++t) ctx->L.half_kick[t] = 0.5 * dt * kAccel / ctx->mass[t];
@@ -549,6 +566,7 @@ md_status profile_impl(md_ctx *ctx, int64_t nsteps, double dt, md_profile_t *out
     md_status rc0 = read_state(ctx);
     if (rc0 != MD_OK) return rc0;
     const long long rebuilds0 = ctx->st_host->rebuilds;
+    touch(ctx);
     const int64_t ne = 4 * nsteps + 2;
     std::vector<cudaEvent_t> ev(ne);
     for (auto &e : ev) CK(cudaEventCreate(&e));
@@ -609,6 +627,20 @@ md_status store_state(md_ctx *ctx, double *pos, double *vel, double *force)
     const size_t n = (size_t)ctx->n;
     if (n == 0) return MD_OK;
     Launch L = ctx->L;
+    if (ctx->host_stage) {
+        // a small system: the kernel writes to pinned host memory and the
+        // host copies from there, instead of a device-to-host copy per array
+        // (which waits in the driver where the caller's memory is pageable)
+        double *h = ctx->host_stage;
+        ctx->fixed_launches += launch_store_state<R>(bufs<R>(ctx), L, pos ? h : nullptr, vel ? h + 3 * n : nullptr,
+                                                     force ? h + 6 * n : nullptr);
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(ctx->stream));
+        if (pos) memcpy(pos, h, 3 * n * sizeof(double));
+        if (vel) memcpy(vel, h + 3 * n, 3 * n * sizeof(double));
+        if (force) memcpy(force, h + 6 * n, 3 * n * sizeof(double));
+        return MD_OK;
+    }
     double *dp = pos ? ctx->stage : nullptr;
     double *dv = vel ? ctx->stage + 3 * n : nullptr;
     double *df = force ? ctx->stage + 6 * n : nullptr;
@@ -707,6 +739,7 @@ std::vector<std::pair<TuneKey, TuneChoice>> g_tune_cache;
 template <class R>
 md_status reevaluate(md_ctx *ctx)
 {
+    touch(ctx);
     const Bufs<R> &B = bufs<R>(ctx);
     Launch L = ctx->L;
     L.use_cond = 0;
@@ -735,6 +768,7 @@ md_status autotune(md_ctx *ctx)
                 return reevaluate<R>(ctx);
             }
     }
+    touch(ctx);
     const Bufs<R> &B = bufs<R>(ctx);
     // block sizes below 256 let the atom-parallel passes fill their last
     // wave of blocks on the GPU
@@ -892,6 +926,7 @@ md_status setup_persistent(md_ctx *ctx)
         ctx->persist = cand[0];
         return MD_OK;
     }
+    touch(ctx);
     const int trial_steps = ctx->L.rebuild_every - 1;
     DevState saved;
     CK(cudaStreamSynchronize(ctx->stream));
@@ -1058,12 +1093,14 @@ md_status force_match_impl(md_ctx *ctx, const double *f_ref, double e_ref, doubl
     // one wait for the energy, the error flags, |g|^2 and the gradient: the
     // kernels take the energy from the device state
     double *out = ctx->adj_host;
-    CK(cudaMemcpyAsync(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
+    if (!ctx->st_current)
+        CK(cudaMemcpyAsync(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(out, ctx->adj_sq, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if (grad)
         CK(cudaMemcpyAsync(out + 1, ctx->adj_kg, sizeof(double) * (size_t)ctx->adj_nknots, cudaMemcpyDeviceToHost,
                            ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    ctx->st_current = true;
     rc = state_errors(ctx);
     if (rc != MD_OK) return rc;
     const double E = ctx->st_host->e_embed + ctx->st_host->e_pair, sq = out[0];
@@ -1097,6 +1134,8 @@ md_status create_impl(md_ctx *ctx, const double *pos, const double *vel, const i
     ctx->skin = pot->skin;
 
     CK(cudaMallocHost((void **)&ctx->st_host, sizeof(DevState)));
+    if (ctx->n > 0 && ctx->n <= kHostStageAtoms)
+        CK(cudaMallocHost((void **)&ctx->host_stage, sizeof(double) * 9 * (size_t)ctx->n));
     if (!alloc_n(ctx, ctx->st, 1) || !alloc_n(ctx, ctx->stage, 9 * (size_t)std::max<int64_t>(ctx->n, 1)) ||
         !alloc_n(ctx, ctx->types_orig, (size_t)std::max<int64_t>(ctx->n, 1)))
         return ctx->fail(MD_ERR_OOM, "device allocation failed");
@@ -1544,6 +1583,7 @@ void md_destroy(md_ctx *ctx)
     dfree_all(ctx);
     if (ctx->st_host) cudaFreeHost(ctx->st_host);
     if (ctx->adj_host) cudaFreeHost(ctx->adj_host);
+    if (ctx->host_stage) cudaFreeHost(ctx->host_stage);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->body_stream) cudaStreamDestroy(ctx->body_stream);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
