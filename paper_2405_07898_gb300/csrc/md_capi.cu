@@ -229,6 +229,8 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
         ok = ok && alloc_n(ctx, B.id[s], n);
         ok = ok && alloc_n(ctx, B.type[s], n);
         ok = ok && alloc_n(ctx, B.shadow[s], n);
+        B.rec32[s] = nullptr;
+        if (sizeof(R) == 8) ok = ok && alloc_n(ctx, B.rec32[s], n);
     }
     ok = ok && alloc_n(ctx, B.cell, n);
     ok = ok && alloc_n(ctx, B.cell_old, n);

@@ -128,6 +128,7 @@ struct Bufs {
     // which its gathers do not use, so the non-coherent texture reads of the
     // coordinates are exact.
     unsigned long long tex_shadow[2];
+    float4 *rec32[2];    // FP64 path: the records' coordinates rounded to FP32
     R *fcache[3];
     int *cell;
     double *center[3];   // cell centres per axis, (c + 1/2) h_d

@@ -156,6 +156,87 @@ __device__ __forceinline__ uint64_t global_ns()
     return t;
 }
 
+// ---- FP64: the listed pairs that are in range, compacted before the FP64 work
+//
+// An FP64 instruction takes its 16 cycles of the SM's pipe whether one lane of
+// the warp needs it or all: with 14 of 26 listed pairs in range (BCC), nearly
+// every column had some lane in range and cost every FP64 operation of a pair.
+// So the columns are first tested in FP32 (records rounded to FP32, a margin
+// for their rounding), the entries that may be in range go to shared memory
+// one behind the other, and the FP64 passes walk those, exact test included.
+// With several lanes per atom the entries found are dealt out anew over the
+// lanes.  The order of an atom's entries is that of its list.
+// 799,496 BCC atoms: density 760 -> 484 us, force 1,267 -> 681 us; the FP64
+// operations alone take about 440 and 580 us of the pipe.
+constexpr int kCompactColumns = 32;  // list columns taken at a time
+
+// Bytes of shared memory a block of the pair passes needs.
+template <class R>
+constexpr size_t compact_bytes(int block, int tpa)
+{
+    return sizeof(R) == 8 ? sizeof(uint32_t) * kCompactColumns * (size_t)(block / tpa) : 0;
+}
+
+extern __shared__ uint32_t compact_smem[];
+
+// Entry k of the compacted columns of the lane's atom.
+struct ListCompact {
+    const uint32_t *p;  // compact_smem + atom of the block
+    int width;          // atoms of the block
+    __device__ __forceinline__ uint32_t operator()(int k) const { return p[k * width]; }
+};
+
+// Upper bound of r_cut^2 in FP32 for the atom at u: twice the rounding bound
+// of r^2 from FP32 records of this size (a partner in range is at most a
+// shift and r_cut farther from its cell's centre).
+__device__ __forceinline__ float compact_bound(const Geom &G, const float4 &u)
+{
+    const float rc = sqrtf(G.rc2_f);
+    const float m = fabsf(u.x) + fabsf(u.y) + fabsf(u.z) + 2.f * (G.h_f[0] + G.h_f[1] + G.h_f[2]) + 6.f * rc;
+    return G.rc2_f + 0x1p-24f * (10.f * rc * m + 16.f * G.rc2_f);
+}
+
+// Entries of columns [k0, min(k0 + kCompactColumns, nn)) of the lane's atom
+// that may be in range, to shared memory; returns their number.  All lanes of
+// the warp must call (nn = 0 without an atom).
+template <int TPA, class List>
+__device__ __forceinline__ int compact_columns(const Geom &G, const float4 *rec, const float4 &ui, float bound, int k0,
+                                               int nn, int l, const List &list, uint32_t *buf, int width)
+{
+    constexpr int U = 4;  // columns in flight per lane
+    const float h[3] = {G.h_f[0], G.h_f[1], G.h_f[2]};
+    const int k1 = min(k0 + kCompactColumns, nn);
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned group = TPA == 1 ? 0u : ((TPA == 32 ? 0u : (1u << (TPA & 31))) - 1u) << (lane & ~(unsigned)(TPA - 1));
+    const unsigned before = (1u << lane) - 1u;
+    // the warp's lanes go round together where they exchange their finds
+    const int kend = TPA == 1 ? k1 : (int)__reduce_max_sync(0xffffffffu, (unsigned)max(k1, 0));
+    int cnt = 0;
+    for (int k = k0; k < kend; k += U * TPA) {
+        uint32_t e[U];
+        float4 u[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) e[q] = (k + l + q * TPA < k1) ? list(k + l + q * TPA) : 0u;
+#pragma unroll
+        for (int q = 0; q < U; ++q) u[q] = (k + l + q * TPA < k1) ? rec[e[q] & kIndexMask] : ui;
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const PairIn<float> p = pair_vector<float>(ui, u[q], entry_shift<float>(e[q], h));
+            const bool in = (k + l + q * TPA < k1) && p.r2 < bound;
+            if (TPA == 1) {
+                if (in) buf[cnt * width] = e[q];
+                cnt += in ? 1 : 0;
+            } else {
+                const unsigned m = __ballot_sync(0xffffffffu, in) & group;
+                if (in) buf[(cnt + __popc(m & before)) * width] = e[q];
+                cnt += __popc(m);
+            }
+        }
+    }
+    __syncwarp();
+    return cnt;
+}
+
 // This lane's part of rho_i = sum over listed j with r < r_cut of f_{t_j}(r_ij)
 // (Eq. 2).
 // In the force pass the list columns of the first round are read before the
@@ -165,13 +246,12 @@ __device__ __forceinline__ uint64_t global_ns()
 template <class R, bool MULTI, int TPA, int U, class List, class Fetch, class Tab>
 __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R rc2, int s, const int *nnb_i,
                                           int cap, int l, const typename V4<R>::T &ui, const List &list,
-                                          const Fetch &fetch, const Tab &tab)
+                                          const Fetch &fetch, const Tab &tab, R rho = (R)0)
 {
     using R4 = typename V4<R>::T;
     const Tables<R> &T = *B.tables;
     const SplineDesc<R> g = MULTI ? T.f[0] : T.fphi;
     const Own<R> own(ui, h);
-    R rho = (R)0;
     // Many lanes per atom (small systems, bound by latency): the columns of
     // the first round are read before the neighbour count is known, as in the
     // force pass.  With few lanes the registers cost more than the wait.
@@ -234,8 +314,8 @@ __device__ __forceinline__ R embed(const Bufs<R> &B, typename V4<R>::T *sw, int 
 // W xx yy zz xy xz yz).
 template <class R, bool MULTI, bool ENERGY, int TPA, int U, class List, class Fetch, class Tab>
 __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, const R (&h)[3], R rc2,
-                                           int s, const int *nnb_i, int l, int ti, const typename V4<R>::T &ui,
-                                           const List &list, const Fetch &fetch, R (&f)[3], R (&e7)[7],
+                                           int s, const int *nnb_i, int cap, int l, int ti,
+                                           const typename V4<R>::T &ui, const List &list, const Fetch &fetch, R (&f)[3], R (&e7)[7],
                                            const Tab &tab)
 {
     using R4 = typename V4<R>::T;
@@ -247,7 +327,7 @@ __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, co
     uint32_t e[U], en[U];
     R4 u[U];
 #pragma unroll
-    for (int q = 0; q < U; ++q) e[q] = (l + q * TPA < L.cap) ? list(l + q * TPA) : 0u;
+    for (int q = 0; q < U; ++q) e[q] = (l + q * TPA < cap) ? list(l + q * TPA) : 0u;
     const int nn = *nnb_i;
 #pragma unroll
     for (int q = 0; q < U; ++q) en[q] = (l + W + q * TPA < nn) ? list(l + W + q * TPA) : 0u;
@@ -347,7 +427,9 @@ __device__ __forceinline__ void integrate(const Bufs<R> &B, const Launch &L, int
         if (MODE == MODE_CLOSE_OPEN) {
             const double dn = fma(v, L.dt, B.d[c][i]);
             B.d[c][i] = dn;
-            reinterpret_cast<R *>(B.shadow[sp ^ 1] + i)[c] = B.uref[c][i] + (R)dn;
+            const R u = B.uref[c][i] + (R)dn;
+            reinterpret_cast<R *>(B.shadow[sp ^ 1] + i)[c] = u;
+            if constexpr (sizeof(R) == 8) reinterpret_cast<float *>(B.rec32[sp ^ 1] + i)[c] = (float)u;
             const float gc = (float)dn;
             d2 += gc * gc;
         }
@@ -367,6 +449,63 @@ __device__ __forceinline__ void force_block_end(const Bufs<R> &B, const Launch &
         block_sums_t<8, R>(v8, B.partials, L.pstride, 1, lo8);
     }
     if (open) block_max_disp(d2max, &B.st->maxdisp2);
+}
+
+// The atom's density and force sums over its whole list: FP32 walks the list,
+// FP64 its columns in range.  All lanes of the warp must call; `active`: the
+// lane has an atom.
+template <class R, bool MULTI, int TPA, int U, class Fetch, class Tab>
+__device__ __forceinline__ R density_atom(const Bufs<R> &B, const Geom &G, const Launch &L, const R (&h)[3], R rc2, int s,
+                                          int sp, int i, int l, bool active, const Fetch &fetch, const Tab &tab)
+{
+    const ListGlobal list{B.list + i, L.ld};
+    if constexpr (sizeof(R) == 8) {
+        const int width = blockDim.x / TPA;
+        uint32_t *buf = compact_smem + threadIdx.x / TPA;
+        const int nn = active ? B.nnb[i] : 0;
+        const typename V4<R>::T ui = active ? B.shadow[sp][i] : mk4<R>(0, 0, 0, 0);
+        const float4 uf = active ? B.rec32[sp][i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float bound = compact_bound(G, uf);
+        const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)nn);
+        R rho = (R)0;
+        for (int k0 = 0; k0 < most; k0 += kCompactColumns) {
+            const int cnt = compact_columns<TPA>(G, B.rec32[sp], uf, bound, k0, nn, l, list, buf, width);
+            rho = density_lane<R, MULTI, TPA, U>(B, h, rc2, s, &cnt, cnt, l, ui, ListCompact{buf, width}, fetch, tab,
+                                                 rho);
+            __syncwarp();  // the buffer is free for the next columns
+        }
+        return rho;
+    } else {
+        return active ? density_lane<R, MULTI, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, B.shadow[sp][i], list, fetch,
+                                                       tab)
+                      : (R)0;
+    }
+}
+
+template <class R, bool MULTI, bool ENERGY, int TPA, int U, class Fetch, class Tab>
+__device__ __forceinline__ void force_atom(const Bufs<R> &B, const Geom &G, const Launch &L, const R (&h)[3], R rc2,
+                                           int s, int sp, int i, int l, int ti, bool active, const Fetch &fetch,
+                                           R (&f)[3], R (&e7)[7], const Tab &tab)
+{
+    const ListGlobal list{B.list + i, L.ld};
+    if constexpr (sizeof(R) == 8) {
+        const int width = blockDim.x / TPA;
+        uint32_t *buf = compact_smem + threadIdx.x / TPA;
+        const int nn = active ? B.nnb[i] : 0;
+        const typename V4<R>::T ui = active ? B.shadow[sp][i] : mk4<R>(0, 0, 0, 0);
+        const float4 uf = active ? B.rec32[sp][i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float bound = compact_bound(G, uf);
+        const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)nn);
+        for (int k0 = 0; k0 < most; k0 += kCompactColumns) {
+            const int cnt = compact_columns<TPA>(G, B.rec32[sp], uf, bound, k0, nn, l, list, buf, width);
+            force_lane<R, MULTI, ENERGY, TPA, U>(B, L, h, rc2, s, &cnt, cnt, l, ti, ui, ListCompact{buf, width}, fetch, f,
+                                                 e7, tab);
+            __syncwarp();
+        }
+    } else if (active) {
+        force_lane<R, MULTI, ENERGY, TPA, U>(B, L, h, rc2, s, B.nnb + i, L.cap, l, ti, B.shadow[sp][i], list, fetch, f,
+                                             e7, tab);
+    }
 }
 
 // ---- L2 prefetch of a warp's streams ----
@@ -410,7 +549,7 @@ __device__ __forceinline__ void prefetch_warp_streams(const Bufs<R> &B, const La
 // ---- atom-parallel schedule ----
 
 // Pairs in flight per lane: the type-dependent path needs more registers a pair.
-template <bool MULTI> struct PairsInFlight {
+template <class R, bool MULTI> struct PairsInFlight {
     static constexpr int density = MULTI ? 2 : 3;
     static constexpr int force = 2;
 };
@@ -419,7 +558,7 @@ template <class R, bool MULTI, bool ENERGY, int TPA, bool TEX>
 __global__ void __launch_bounds__(256) k_density(Bufs<R> B, Geom G, Launch L)
 {
     using R4 = typename V4<R>::T;
-    constexpr int U = PairsInFlight<MULTI>::density;
+    constexpr int U = PairsInFlight<R, MULTI>::density;
     R h[3];
     load_h<R>(G, h);
     const DevState *st = B.st;
@@ -432,18 +571,13 @@ __global__ void __launch_bounds__(256) k_density(Bufs<R> B, Geom G, Launch L)
     const bool active = i < L.n;
     const int ti = (MULTI && active) ? B.type[s][i] : 0;
     const R rc2 = g_rc2<R>(G);
-    R rho = (R)0;
-    if (active) {
-        if constexpr (TEX)
-            rho = density_lane<R, MULTI, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, sw[i],
-                                                 ListGlobal{B.list + i, L.ld},
-                                                 TexFetch{(cudaTextureObject_t)B.tex_shadow[sp]},
-                                                 TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
-        else
-            rho = density_lane<R, MULTI, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, sw[i],
-                                                 ListGlobal{B.list + i, L.ld}, GlobalFetch<R>{sw},
-                                                 TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
-    }
+    const TabGlobal<R> tab{B.coef2, B.coef_f, B.coef_d};
+    R rho;
+    if constexpr (TEX)
+        rho = density_atom<R, MULTI, TPA, U>(B, G, L, h, rc2, s, sp, i, l, active,
+                                             TexFetch{(cudaTextureObject_t)B.tex_shadow[sp]}, tab);
+    else
+        rho = density_atom<R, MULTI, TPA, U>(B, G, L, h, rc2, s, sp, i, l, active, GlobalFetch<R>{sw}, tab);
     rho = lane_sum<TPA>(rho);
     R e_embed = (R)0;
     if (active && l == 0) e_embed = embed<R>(B, sw, i, ti, rho);
@@ -457,7 +591,7 @@ template <class R, bool MULTI, int MODE, bool ENERGY, int TPA>
 __global__ void __launch_bounds__(256) k_force(Bufs<R> B, Geom G, Launch L)
 {
     using R4 = typename V4<R>::T;
-    constexpr int U = PairsInFlight<MULTI>::force;
+    constexpr int U = PairsInFlight<R, MULTI>::force;
     R h[3];
     load_h<R>(G, h);
     const DevState *st = B.st;
@@ -472,9 +606,8 @@ __global__ void __launch_bounds__(256) k_force(Bufs<R> B, Geom G, Launch L)
     const R rc2 = g_rc2<R>(G);
     R f[3] = {0, 0, 0};
     R e7[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (active)
-        force_lane<R, MULTI, ENERGY, TPA, U>(B, L, h, rc2, s, B.nnb + i, l, ti, sw[i], ListGlobal{B.list + i, L.ld},
-                                             GlobalFetch<R>{sw}, f, e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+    force_atom<R, MULTI, ENERGY, TPA, U>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f, e7,
+                                         TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
 #pragma unroll
     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
     double ke = 0.0;
@@ -700,10 +833,10 @@ void density_tpa_fetch(const Bufs<R> &B, const Geom &G, const Launch &L)
 {
     dim3 g(L.nb_d), b(L.block_d);
     switch (L.tpa_d) {
-    case 1: k_density<R, MULTI, ENERGY, 1, TEX><<<g, b, 0, L.stream>>>(B, G, L); break;
-    case 2: k_density<R, MULTI, ENERGY, 2, TEX><<<g, b, 0, L.stream>>>(B, G, L); break;
-    case 4: k_density<R, MULTI, ENERGY, 4, TEX><<<g, b, 0, L.stream>>>(B, G, L); break;
-    default: k_density<R, MULTI, ENERGY, 8, TEX><<<g, b, 0, L.stream>>>(B, G, L); break;
+    case 1: k_density<R, MULTI, ENERGY, 1, TEX><<<g, b, compact_bytes<R>(L.block_d, 1), L.stream>>>(B, G, L); break;
+    case 2: k_density<R, MULTI, ENERGY, 2, TEX><<<g, b, compact_bytes<R>(L.block_d, 2), L.stream>>>(B, G, L); break;
+    case 4: k_density<R, MULTI, ENERGY, 4, TEX><<<g, b, compact_bytes<R>(L.block_d, 4), L.stream>>>(B, G, L); break;
+    default: k_density<R, MULTI, ENERGY, 8, TEX><<<g, b, compact_bytes<R>(L.block_d, 8), L.stream>>>(B, G, L); break;
     }
 }
 
@@ -726,10 +859,10 @@ void force_tpa(const Bufs<R> &B, const Geom &G, const Launch &L)
 {
     dim3 g(L.nb_f), b(L.block_f);
     switch (L.tpa_f) {
-    case 1: k_force<R, MULTI, MODE, ENERGY, 1><<<g, b, 0, L.stream>>>(B, G, L); break;
-    case 2: k_force<R, MULTI, MODE, ENERGY, 2><<<g, b, 0, L.stream>>>(B, G, L); break;
-    case 4: k_force<R, MULTI, MODE, ENERGY, 4><<<g, b, 0, L.stream>>>(B, G, L); break;
-    default: k_force<R, MULTI, MODE, ENERGY, 8><<<g, b, 0, L.stream>>>(B, G, L); break;
+    case 1: k_force<R, MULTI, MODE, ENERGY, 1><<<g, b, compact_bytes<R>(L.block_f, 1), L.stream>>>(B, G, L); break;
+    case 2: k_force<R, MULTI, MODE, ENERGY, 2><<<g, b, compact_bytes<R>(L.block_f, 2), L.stream>>>(B, G, L); break;
+    case 4: k_force<R, MULTI, MODE, ENERGY, 4><<<g, b, compact_bytes<R>(L.block_f, 4), L.stream>>>(B, G, L); break;
+    default: k_force<R, MULTI, MODE, ENERGY, 8><<<g, b, compact_bytes<R>(L.block_f, 8), L.stream>>>(B, G, L); break;
     }
 }
 

@@ -96,7 +96,7 @@ template <class R, bool MULTI, int TPA>
 __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long long nsteps, PersistScratch *ps)
 {
     using R4 = typename V4<R>::T;
-    constexpr int UD = PairsInFlight<MULTI>::density, UF = PairsInFlight<MULTI>::force;
+    constexpr int UD = PairsInFlight<R, MULTI>::density, UF = PairsInFlight<R, MULTI>::force;
     DevState *st = B.st;
     unsigned *err = &st->error;
     unsigned long long target = 0;  // of the grid barriers
@@ -174,10 +174,8 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                 const int i = tile * width + threadIdx.x / TPA;
                 const bool active = i < n;
                 const int ti = (MULTI && active) ? B.type[s][i] : 0;
-                R rho = (R)0;
-                if (active)
-                    rho = density_lane<R, MULTI, TPA, UD>(B, h, rc2, s, B.nnb + i, L.cap, l, sw[i], ListGlobal{B.list + i, L.ld},
-                                                          GlobalFetch<R>{sw}, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+                R rho = density_atom<R, MULTI, TPA, UD>(B, G, L, h, rc2, s, sp, i, l, active, GlobalFetch<R>{sw},
+                                                        TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
                 rho = lane_sum<TPA>(rho);
                 if (active && l == 0) e_embed += embed<R>(B, sw, i, ti, rho);
             }
@@ -201,7 +199,6 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                 const int ti = (MULTI && active) ? B.type[s][i] : 0;
                 R f[3] = {0, 0, 0};
                 float d2 = 0.f;
-                const ListGlobal list{B.list + i, L.ld};
                 // the integration's inputs into L1 while the pair loop runs
                 if (active && l == 0) {
 #pragma unroll
@@ -212,16 +209,14 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                     }
                 }
                 if (last) {
-                    if (active)
-                        force_lane<R, MULTI, true, TPA, UF>(B, L, h, rc2, s, B.nnb + i, l, ti, sw[i], list,
-                                                            GlobalFetch<R>{sw}, f, e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+                    force_atom<R, MULTI, true, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
+                                                        e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
 #pragma unroll
                     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
                     if (active) integrate<R, MODE_CLOSE, true, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
                 } else {
-                    if (active)
-                        force_lane<R, MULTI, false, TPA, UF>(B, L, h, rc2, s, B.nnb + i, l, ti, sw[i], list,
-                                                             GlobalFetch<R>{sw}, f, e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+                    force_atom<R, MULTI, false, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
+                                                         e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
 #pragma unroll
                     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
                     if (active) integrate<R, MODE_CLOSE_OPEN, false, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
@@ -274,7 +269,7 @@ int persistent_grid(const Launch &L, int tpa, int block)
 {
     const void *fn = L.multi ? steps_kernel<R, true>(tpa) : steps_kernel<R, false>(tpa);
     int per_sm = 0, dev = 0, nsm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, compact_bytes<R>(block, tpa)) != cudaSuccess ||
         cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm <= 0)
         return 0;
@@ -296,7 +291,8 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
     void *args[] = {&b, &g, &l, &ns, &p};
     cudaError_t e = cudaMemsetAsync(&ps->arrive, 0, sizeof(ps->arrive), L.stream);
     if (e != cudaSuccess) return e;
-    return cudaLaunchCooperativeKernel(fn, dim3(sched.grid), dim3(sched.block), args, 0, L.stream);
+    return cudaLaunchCooperativeKernel(fn, dim3(sched.grid), dim3(sched.block), args,
+                                       compact_bytes<R>(sched.block, sched.tpa), L.stream);
 }
 
 template int persistent_grid<float>(const Launch &, int, int);

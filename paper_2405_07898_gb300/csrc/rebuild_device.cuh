@@ -197,6 +197,7 @@ __device__ __forceinline__ void permute_atom(const Bufs<R> &B, const Geom &G, in
     B.shadow[sp][p] = mk4<R>(u[0], u[1], u[2], (R)0);
     B.screen[0][p] = (float)X0;
     if constexpr (sizeof(R) == 8) {
+        B.rec32[sp][p] = make_float4((float)u[0], (float)u[1], (float)u[2], 0.f);
         B.screen[1][p] = (float)u[1];
         B.screen[2][p] = (float)u[2];
     }
@@ -577,6 +578,7 @@ __device__ __forceinline__ float open_atom(const Bufs<R> &B, const Launch &L, in
     }
     R u0 = B.uref[0][i] + (R)dn[0], u1 = B.uref[1][i] + (R)dn[1], u2 = B.uref[2][i] + (R)dn[2];
     B.shadow[sp ^ 1][i] = mk4<R>(u0, u1, u2, (R)0);
+    if constexpr (sizeof(R) == 8) B.rec32[sp ^ 1][i] = make_float4((float)u0, (float)u1, (float)u2, 0.f);
     float fx = (float)dn[0], fy = (float)dn[1], fz = (float)dn[2];
     return fx * fx + fy * fy + fz * fz;
 }
