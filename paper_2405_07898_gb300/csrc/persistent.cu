@@ -51,8 +51,8 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
 // first and relaxed polls before one acquire load, 11.26 with relaxed polls
 // and a fence, 10.45 so.)
 // Returns false once a wait of the launch has timed out (a block that waits
-// looks at the error word every 64th poll; one that gave up arrives no more,
-// so nobody passes a later barrier).
+// reads the clock every 4th poll and the error word every 64th; one that gave
+// up arrives no more, so nobody passes a later barrier).
 __device__ __forceinline__ bool grid_barrier(PersistScratch *ps, unsigned *err, uint64_t wait_ns,
                                              unsigned long long &target)
 {
@@ -66,7 +66,9 @@ __device__ __forceinline__ bool grid_barrier(PersistScratch *ps, unsigned *err, 
             const uint64_t t0 = global_ns();
             unsigned spins = 0;
             while (ld_acquire(&ps->arrive) < target) {
-                if ((++spins & 63u) == 0 && ((ld_acquire(err) & ERR_TIMEOUT) || global_ns() - t0 > wait_ns)) {
+                ++spins;
+                if (((spins & 3u) == 0 && global_ns() - t0 > wait_ns) ||
+                    ((spins & 63u) == 0 && (ld_acquire(err) & ERR_TIMEOUT))) {
                     atomicOr(err, ERR_TIMEOUT);
                     good = 0;
                     break;
