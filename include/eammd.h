@@ -138,10 +138,11 @@ enum { MD_PERSIST_AUTO = 0, MD_PERSIST_OFF = 1, MD_PERSIST_ON = 2 };
  *   wait_limit_us    longest device-side wait (a grid barrier of the single
  *                    launch) before the kernel gives up and raises
  *                    MD_ERR_TIMEOUT; 0 = 1 s.
- *   batch_schedule   batches only: 0 = threads per block and resident
- *                    blocks per SM timed at md_batch_create (unless
- *                    lanes_per_atom > 0, which takes 512 x 1); 1..5 =
- *                    512 x 1, 256 x 2, 256 x 3, 1024 x 1, 512 x 2.
+ *   batch_schedule   batches only: 0 = threads per block, resident blocks
+ *                    per SM and blocks per replica timed at md_batch_create
+ *                    (unless lanes_per_atom > 0, which takes 512 x 1); 1..5 =
+ *                    512 x 1, 256 x 2, 256 x 3, 1024 x 1, 512 x 2, one block
+ *                    per replica.
  *   half_list        0: every atom lists all its neighbours and each pair is
  *                    evaluated from both ends (the default).  1: the
  *                    force-symmetry form (Section "Additional Acceleration"): each pair
@@ -328,9 +329,10 @@ md_status md_bin_cells_noalloc(const double box[3], double r_list, int64_t n, co
 /* ---- batches: many independent systems in one persistent launch ----
  * The batching form of the method: hundreds of periodic systems ("replicas")
  * of uneven size, each with its own box and one-type potential, advanced
- * together.  One thread block runs all phases of all steps of a replica
- * (list rebuild, density, force and integration) with block-level barriers
- * only; blocks take replicas largest first.  Mixed precision only (FP32
+ * together.  One thread block, or a cluster of blocks where replicas are few,
+ * runs all phases of all steps of a replica (list rebuild, density, force and
+ * integration) with barriers among its own threads only; replicas are taken
+ * costliest first.  Mixed precision only (FP32
  * pair arithmetic, FP64 positions, velocities and sums), the same
  * arithmetic and list rules as a single context. */
 typedef struct md_batch md_batch;

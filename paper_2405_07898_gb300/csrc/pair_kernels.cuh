@@ -129,6 +129,8 @@ struct TabGlobal {
     const typename V4<R>::T *coef2;
     const typename V4<R>::T *coef_f;  // f rows alone: more intervals per cache line
     const typename V4<R>::T *coef_d;  // f' and phi' rows
+    // interval of r (tables of up to kMaxFusedIntervals intervals)
+    __device__ __forceinline__ int interval(const SplineDesc<R> &g, R r, R &t) const { return segment_fused(g, r, t); }
     __device__ __forceinline__ typename V4<R>::T f(int kk) const { return coef_f[kk]; }
     __device__ __forceinline__ void fphi(int kk, typename V4<R>::T &cf, typename V4<R>::T &cp) const
     {
@@ -285,7 +287,7 @@ __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R r
                     rho += val;
                 } else {
                     R t;
-                    const int kk = segment_fused(g, r, t);
+                    const int kk = tab.interval(g, r, t);
                     const R4 c = tab.f(kk);
                     rho += fma(t, fma(t, fma(t, c.w, c.z), c.y), c.x);
                 }
@@ -359,7 +361,7 @@ __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, co
                     fdi = (tj == ti) ? fdj : spline_r_der(T.f[ti], B.coef, r);
                 } else {
                     R t;
-                    const int kk = segment_fused(g, r, t);
+                    const int kk = tab.interval(g, r, t);
                     if (ENERGY) {
                         R4 cf, cp;
                         tab.fphi(kk, cf, cp);

@@ -48,6 +48,19 @@ __device__ __forceinline__ int cell_index(double x, double inv, float inv_f, int
     return cell_index_exact(x, inv, n);
 }
 
+// Slot of an atom in its cell (arrival order): one atomic per distinct cell
+// among the warp's active lanes (atoms in cell order mostly share cells); the
+// lanes of a cell take consecutive slots from it in lane order.
+__device__ __forceinline__ int cell_slot(int *count, int cell)
+{
+    const unsigned peers = __match_any_sync(__activemask(), cell);
+    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
+    int base = 0;
+    if (lane == leader) base = atomicAdd(&count[cell], __popc(peers));
+    base = __shfl_sync(peers, base, leader);
+    return base + __popc(peers & ((1u << lane) - 1u));
+}
+
 // Periodic image of x = xr + d on periodic axes: kept when already in
 // [0, L), else x - L floor(x / L); then bin: c_d = floor(x_d n_d/L_d) clamped
 // to [0, n_d - 1].  The box test compares bit patterns (non-negative doubles
@@ -75,15 +88,7 @@ __device__ __forceinline__ void bin_atom(const Bufs<R> &B, const Geom &G, int s,
     if (!finite) atomicOr(&B.st->error, ERR_NONFINITE);
     int cell = (c[2] * G.ncell[1] + c[1]) * G.ncell[0] + c[0];
     B.cell_old[i] = cell;
-    // one atomic per distinct cell among the warp's active lanes (atoms in
-    // cell order mostly share cells); the lanes of a cell take consecutive
-    // slots from it in lane order
-    const unsigned peers = __match_any_sync(__activemask(), cell);
-    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(&B.count[cell], __popc(peers));
-    base = __shfl_sync(peers, base, leader);
-    B.slot[i] = base + __popc(peers & ((1u << lane) - 1u));
+    B.slot[i] = cell_slot(B.count, cell);
 }
 
 // Sum over the block of one int per thread; every thread returns it.  All
@@ -327,20 +332,19 @@ __device__ __forceinline__ float screen_margin(const Geom &G, float x, float y, 
 // only the neighbours q whose pair vector x_q - x_p lies in the upper half
 // space (upper_half).  Every atom's neighbourhood is close to centrally
 // symmetric, so each lists about half its neighbours.
-template <class R>
-__device__ __forceinline__ int list_atom(const Bufs<R> &B, const Geom &G, int s, int p, int ld, int cap,
-                                         bool half = false)
+//
+// `xr`: exact positions, `cell_of`: the atoms' cells, lp: column 0 of atom p.
+__device__ __forceinline__ int list_walk(const Geom &G, const Screen &sc, const double *const (&xr)[3],
+                                         const int *cell_of, const int *cell_start, int p, uint32_t *lp, int ld, int cap,
+                                         bool half)
 {
     int cnt = 0;
-    const double *const xr[3] = {B.xr[s][0], B.xr[s][1], B.xr[s][2]};
-    const Screen sc = screen_of(B);
     const int nx = G.ncell[0], ny = G.ncell[1], nz = G.ncell[2];
-    const int cell = B.cell[p];
+    const int cell = cell_of[p];
     const int cx = cell % nx, cy = (cell / nx) % ny, cz = cell / (nx * ny);
     const float px = sc.x[p], py = sc.y[p], pz = sc.z[p];
     const float margin = screen_margin(G, px, py, pz);
     const F2 hi = f2(-(G.rl2_f + margin), -(G.rl2_f + margin)), band = f2(2.f * margin, 2.f * margin);
-    uint32_t *lp = B.list + p;
     const bool open_x = G.open_mask & 1, open_y = (G.open_mask >> 1) & 1, open_z = (G.open_mask >> 2) & 1;
 #pragma unroll 1
     for (int row = 0; row < 9; ++row) {
@@ -354,7 +358,7 @@ __device__ __forceinline__ int list_atom(const Bufs<R> &B, const Geom &G, int s,
             if (open_y) continue;
             ey += (ey < 0) ? ny : -ny;
         }
-        const int *cs = B.cell_start + (ez * ny + ey) * nx;
+        const int *cs = cell_start + (ez * ny + ey) * nx;
         const float oy = (float)dy * G.h_f[1] - py, oz = (float)dz * G.h_f[2] - pz;
         const F2 oy2 = f2(oy, oy), oz2 = f2(oz, oz);
         // cells cx - 1, cx, cx + 1: one run of atoms, with the parts beyond an
@@ -432,6 +436,15 @@ __device__ __forceinline__ int list_atom(const Bufs<R> &B, const Geom &G, int s,
             }
         }
     }
+    return cnt;
+}
+
+template <class R>
+__device__ __forceinline__ int list_atom(const Bufs<R> &B, const Geom &G, int s, int p, int ld, int cap,
+                                         bool half = false)
+{
+    const double *const xr[3] = {B.xr[s][0], B.xr[s][1], B.xr[s][2]};
+    const int cnt = list_walk(G, screen_of(B), xr, B.cell, B.cell_start, p, B.list + p, ld, cap, half);
     B.nnb[p] = min(cnt, cap);
     if (cnt > cap) atomicOr(&B.st->error, ERR_LIST_OVERFLOW);
     return cnt;
