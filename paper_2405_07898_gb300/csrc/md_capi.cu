@@ -725,11 +725,13 @@ void set_sched(md_ctx *ctx, PassSched d, PassSched f)
     L.nb_f = blocks_for_host((int64_t)L.n * f.tpa, L.block_f);
 }
 
-// Choices of the autotuner, per (precision, type path, size bucket), kept for
+// Choices of the autotuner, per (precision, type path, size bucket, list
+// capacity: the FCC slab's 54 neighbours per atom take another schedule than
+// BCC's 26), kept for
 // the life of the process so that every context of the same shape runs the
 // same schedule (and gives bitwise identical results).
 struct TuneKey {
-    int precision, multi, bucket;
+    int precision, multi, bucket, cap;
 };
 struct TuneChoice {
     PassSched d, f;
@@ -761,11 +763,12 @@ md_status autotune(md_ctx *ctx)
 {
     int bucket = 0;
     for (int64_t m = ctx->n; m > 1; m >>= 1) ++bucket;
-    TuneKey key{ctx->precision, ctx->L.multi, bucket};
+    TuneKey key{ctx->precision, ctx->L.multi, bucket, ctx->L.cap};
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         for (auto &e : g_tune_cache)
-            if (e.first.precision == key.precision && e.first.multi == key.multi && e.first.bucket == key.bucket) {
+            if (e.first.precision == key.precision && e.first.multi == key.multi && e.first.bucket == key.bucket &&
+                e.first.cap == key.cap) {
                 set_sched(ctx, e.second.d, e.second.f);
                 return reevaluate<R>(ctx);
             }
