@@ -135,7 +135,7 @@ __device__ __forceinline__ void warp_max_disp(float d2, unsigned *dst)
 // The replica's spline rows, for tables of any size (segment_fused takes up to
 // kMaxFusedIntervals intervals).
 struct TabBatch : TabGlobal<float> {
-    __device__ __forceinline__ explicit TabBatch(const Bufs<float> &B) : TabGlobal<float>{B.coef2, B.coef_f, B.coef_d} {}
+    __device__ __forceinline__ explicit TabBatch(const Bufs<float> &B) : TabGlobal<float>(B) {}
     __device__ __forceinline__ int interval(const SplineDesc<float> &g, float r, float &t) const
     {
         return g.nint > kMaxFusedIntervals ? segment(g, r, t) : segment_fused(g, r, t);
@@ -151,7 +151,7 @@ __device__ __forceinline__ void force_phase(const Replica &R, const float (&h)[3
     const float4 *sw = B.shadow[sp];
     for (int i = i0 + (int)threadIdx.x; i < i1; i += blockDim.x) {
         float f[3] = {0.f, 0.f, 0.f}, e7[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, d2 = 0.f;
-        force_lane<float, false, ENERGY, 1, kBatchForcePairs>(B, R.L, h, rc2, s, B.nnb + i, R.L.cap, 0, 0, sw[i],
+        force_lane<float, KIND_ONE, ENERGY, 1, kBatchForcePairs>(B, R.L, h, rc2, s, B.nnb + i, R.L.cap, 0, 0, sw[i],
                                                               ListGlobal{B.list + i, R.L.ld}, GlobalFetch<float>{sw}, f,
                                                               e7, TabBatch(B));
         integrate<float, MODE, ENERGY, 1>(B, R.L, s, sp, i, 0, 0, f, ke, d2);
@@ -218,7 +218,7 @@ __device__ void run_replica(const BatchArgs &A, BatchSmem &S, int r, int rank, i
         float4 *sw = B.shadow[sp];
         float e_emb = 0.f;
         for (int i = i0 + tid; i < i1; i += nt) {
-            const float rho = density_lane<float, false, 1, kBatchDensityPairs>(
+            const float rho = density_lane<float, KIND_ONE, 1, kBatchDensityPairs>(
                 B, h, rc2, s, B.nnb + i, R.L.cap, 0, sw[i], ListGlobal{B.list + i, R.L.ld}, GlobalFetch<float>{sw},
                 TabBatch(B));
             e_emb += embed<float>(B, sw, i, 0, rho);
@@ -670,7 +670,7 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
              balloc_n(b, B.fcache[a], N);
     for (int s = 0; s < 2; ++s) ok = ok && balloc_n(b, B.id[s], N) && balloc_n(b, B.type[s], N) && balloc_n(b, B.shadow[s], N);
     ok = ok && balloc_n(b, B.cell, N) && balloc_n(b, B.cell_old, N) && balloc_n(b, B.slot, N) &&
-         balloc_n(b, B.cell_atoms, N) && balloc_n(b, B.cell_ids, N) && balloc_n(b, B.screen[0], N) && balloc_n(b, B.nnb, N);
+         balloc_n(b, B.cell_atoms, N) && balloc_n(b, B.cell_ids, N) && balloc_n(b, B.screen[0], N) && balloc_n(b, B.type8, N) && balloc_n(b, B.nnb, N);
     ok = ok && balloc_n(b, B.count, (size_t)cell_off) && balloc_n(b, B.cell_start, (size_t)cs_off);
     ok = ok && balloc_n(b, B.list, (size_t)cap * (size_t)atom_off);
     size_t ncenter = 0;
@@ -721,6 +721,7 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
         V.cell_atoms += at.atom;
         V.cell_ids += at.atom;
         V.screen[0] += at.atom;
+        V.type8 += at.atom;
         V.nnb += at.atom;
         V.count += at.cell;
         V.cell_start += at.cs;

@@ -232,6 +232,7 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
         B.rec32[s] = nullptr;
         if (sizeof(R) == 8) ok = ok && alloc_n(ctx, B.rec32[s], n);
     }
+    ok = ok && alloc_n(ctx, B.type8, n);
     ok = ok && alloc_n(ctx, B.cell, n);
     ok = ok && alloc_n(ctx, B.cell_old, n);
     ok = ok && alloc_n(ctx, B.slot, n);
@@ -256,8 +257,9 @@ bool alloc_buffers(md_ctx *ctx, const std::vector<double> &rows, const std::vect
     if (!ok) return false;
     B.coef = coef;
     B.coef2 = coef2;
-    B.coef_d = tables.fused ? coef2 + 2 * (size_t)tables.fphi.nint : coef2;
-    B.coef_f = tables.fused ? coef2 + 4 * (size_t)tables.fphi.nint : coef2;
+    const size_t nint = (size_t)tables.fphi.nint, npair = (size_t)tables.ntypes * (tables.ntypes + 1) / 2;
+    B.coef_d = tables.fused == 1 ? coef2 + 2 * nint : coef2;
+    B.coef_f = tables.fused == 1 ? coef2 + 4 * nint : (tables.fused == 2 ? coef2 + 4 * npair * nint : coef2);
     B.tables = tab;
     B.st = ctx->st;
     auto upload = [](R4 *dst_dev, const std::vector<double> &src) -> bool {
@@ -706,6 +708,31 @@ md_status build_tables(md_ctx *ctx, const md_potential *pot, std::vector<double>
         for (int k = 0; k < f0.n - 1; ++k)
             for (int c = 0; c < 4; ++c) rows2.push_back(rows[4 * ((size_t)tab.f[0].offset + k) + c]);
     }
+    // several types whose f and phi all share a knot grid: per type pair the
+    // rows of the three derivatives that its force needs, then the f rows
+    bool shared = pot->ntypes > 1;
+    auto same = [&](const md_spline &a) { return a.n == f0.n && a.x0 == f0.x0 && a.dx == f0.dx; };
+    for (int t = 0; t < pot->ntypes; ++t) shared = shared && same(pot->f[t]);
+    for (int q = 0; q < npair; ++q) shared = shared && same(pot->phi[q]);
+    if (shared) {
+        tab.fused = 2;
+        tab.fphi = tab.f[0];
+        tab.fphi.offset = 0;
+        for (int a = 0, q = 0; a < pot->ntypes; ++a)
+            for (int b = a; b < pot->ntypes; ++b, ++q)
+                for (int k = 0; k < f0.n - 1; ++k) {
+                    for (const auto &d : {tab.f[a], tab.f[b], tab.phi[q]}) {
+                        const double *c = &rows[4 * ((size_t)d.offset + k)];
+                        rows2.push_back(c[1]);
+                        rows2.push_back(2.0 * c[2]);
+                        rows2.push_back((double)((R)3 * (R)c[3]));
+                    }
+                    for (int z = 0; z < 7; ++z) rows2.push_back(0.0);
+                }
+        for (int t = 0; t < pot->ntypes; ++t)
+            for (int k = 0; k < f0.n - 1; ++k)
+                for (int c = 0; c < 4; ++c) rows2.push_back(rows[4 * ((size_t)tab.f[t].offset + k) + c]);
+    }
     return MD_OK;
 }
 
@@ -1122,9 +1149,9 @@ md_status create_impl(md_ctx *ctx, const double *pos, const double *vel, const i
     Tables<R> tab;
     md_status trc = build_tables<R>(ctx, pot, rows, rows2, tab);
     if (trc != MD_OK) return trc;
-    ctx->L.multi = tab.fused && tab.fphi.nint <= kMaxFusedIntervals ? 0 : 1;
+    ctx->L.multi = tab.fused && tab.fphi.nint <= kMaxFusedIntervals ? (tab.fused == 2 ? 2 : 0) : 1;
     ctx->L.nint_fused = tab.fused ? tab.fphi.nint : 0;
-    if (ctx->opt.half_list && (ctx->precision != MD_PRECISION_MIXED || !tab.fused))
+    if (ctx->opt.half_list && (ctx->precision != MD_PRECISION_MIXED || tab.fused != 1))
         return ctx->fail(MD_ERR_ARG, "half_list takes mixed precision and one atom type whose f and phi share a knot grid");
     ctx->L.half = ctx->opt.half_list ? 1 : 0;
     ctx->shapes.clear();

@@ -89,8 +89,8 @@ struct SplineDesc {
 template <class R>
 struct Tables {
     int ntypes;
-    int fused;             // 1: one type whose f and phi share a knot grid (fphi)
-    SplineDesc<R> fphi;    // grid of the fused rows: coef2[2k] = f, coef2[2k+1] = phi
+    int fused;             // f and phi of all types share a knot grid (fphi): 1 one type, 2 several
+    SplineDesc<R> fphi;    // that grid; one type: coef2[2k] = f, coef2[2k+1] = phi
     SplineDesc<R> F[kMaxTypes], f[kMaxTypes], phi[kMaxPairs];
 };
 
@@ -119,6 +119,7 @@ struct Bufs {
     double *v[2][3];
     int *id[2];
     int *type[2];
+    uint8_t *type8;      // types in the current order, a byte each (gathered per pair)
     R *uref[3];
     R4 *shadow[2];
     // texture objects over shadow[0] and shadow[1] (FP32 records only; 0 =
@@ -155,9 +156,10 @@ struct Bufs {
     DevState *st;
     const R4 *coef;
     const R4 *coef2;     // fused f | phi rows (single-type fast path)
-    const R4 *coef_f;    // the f rows alone (coef2 + 4 nint), read by the density pass
-    const R4 *coef_d;    // rows (f': b, 2c, 3d; phi': b, 2c, 3d; 0, 0) (coef2 + 2 nint), read by the
-                         // force pass when it forms no energies
+    const R4 *coef_f;    // the f rows alone, type after type, read by the density pass
+    const R4 *coef_d;    // read by the force pass when it forms no energies.  One type: rows (f': b,
+                         // 2c, 3d; phi': b, 2c, 3d; 0, 0).  Several: per type pair a <= b, rows of 16
+                         // words (b, 2c, 3d of f_a', f_b', phi'; zeros)
     const Tables<R> *tables;
 };
 
@@ -176,7 +178,8 @@ struct Launch {
     int nb_f;       // blocks of the force pass
     int pstride;    // stride between energy slots in partials (>= nb_d, nb_f)
     int nint_fused; // intervals of the fused f|phi table (0: not fused)
-    int multi;      // general type-dependent path (several types or unfused tables)
+    int multi;      // kind of the tables (pair_kernels.cuh): 0 one type with fused tables, 1 any,
+                    // 2 several types whose f and phi share one knot grid
     int half;       // 1: half lists (each pair once, j < i ends added through acc_*)
     int ntypes;
     int rebuild_every;

@@ -20,6 +20,10 @@
 namespace eammd {
 namespace {
 
+// Kinds of spline tables: one type whose f and phi share a knot grid; any
+// tables; several types whose f and phi all share one grid.
+enum TableKind { KIND_ONE = 0, KIND_ANY = 1, KIND_TYPES = 2 };
+
 template <class R> struct PairIn {
     R dx, dy, dz, r2;
 };
@@ -128,13 +132,33 @@ template <class R>
 struct TabGlobal {
     const typename V4<R>::T *coef2;
     const typename V4<R>::T *coef_f;  // f rows alone: more intervals per cache line
-    const typename V4<R>::T *coef_d;  // f' and phi' rows
+    const typename V4<R>::T *coef_d;  // f' and phi' rows (of a type pair: slopes_types)
+    const uint8_t *type8;             // types of the atoms, where there are several
+    __device__ __forceinline__ explicit TabGlobal(const Bufs<R> &B)
+        : coef2(B.coef2), coef_f(B.coef_f), coef_d(B.coef_d), type8(B.type8)
+    {
+    }
     // interval of r (tables of up to kMaxFusedIntervals intervals)
     __device__ __forceinline__ int interval(const SplineDesc<R> &g, R r, R &t) const { return segment_fused(g, r, t); }
     __device__ __forceinline__ typename V4<R>::T f(int kk) const { return coef_f[kk]; }
     __device__ __forceinline__ void fphi(int kk, typename V4<R>::T &cf, typename V4<R>::T &cp) const
     {
         load_row2<R>(coef2 + 2 * kk, cf, cp);
+    }
+    // f' of types ti and tj and phi' of the pair at t, row kk of the nint of
+    // each type pair: 16 words, nine in use (b, 2c, 3d of f_a, f_b and phi,
+    // a <= b), by one 256-bit load and one word
+    __device__ __forceinline__ void slopes_types(int ntypes, int nint, int ti, int tj, int kk, R t, R &fi, R &fj,
+                                                 R &pd) const
+    {
+        typename V4<R>::T a, b;
+        const typename V4<R>::T *row = coef_d + 4 * ((size_t)pair_index(ntypes, ti, tj) * nint + kk);
+        load_row2<R>(row, a, b);
+        const R p3 = reinterpret_cast<const R *>(row)[8];
+        const R fa = fma(t, fma(t, a.z, a.y), a.x), fb = fma(t, fma(t, b.y, b.x), a.w);
+        fi = ti <= tj ? fa : fb;
+        fj = ti <= tj ? fb : fa;
+        pd = fma(t, fma(t, p3, b.w), b.z);
     }
     // f' and phi' at t
     __device__ __forceinline__ void slopes(int kk, R t, R &fd, R &pd) const
@@ -245,14 +269,14 @@ __device__ __forceinline__ int compact_columns(const Geom &G, const float4 *rec,
 // neighbour count is known (every column below cap lies inside the list);
 // while a round is computed, the next round's records and the columns of the
 // round after are in flight.  Columns at or beyond nn never address a record.
-template <class R, bool MULTI, int TPA, int U, class List, class Fetch, class Tab>
+template <class R, int KIND, int TPA, int U, class List, class Fetch, class Tab>
 __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R rc2, int s, const int *nnb_i,
                                           int cap, int l, const typename V4<R>::T &ui, const List &list,
                                           const Fetch &fetch, const Tab &tab, R rho = (R)0)
 {
     using R4 = typename V4<R>::T;
     const Tables<R> &T = *B.tables;
-    const SplineDesc<R> g = MULTI ? T.f[0] : T.fphi;
+    const SplineDesc<R> g = T.fphi;
     const Own<R> own(ui, h);
     // Many lanes per atom (small systems, bound by latency): the columns of
     // the first round are read before the neighbour count is known, as in the
@@ -280,14 +304,15 @@ __device__ __forceinline__ R density_lane(const Bufs<R> &B, const R (&h)[3], R r
             if ((q == 0 || k + q * TPA < nn) && within(p.r2, rc2)) {
                 R rinv, r;
                 inv_r(p.r2, rinv, r);
-                if (MULTI) {
+                if (KIND == KIND_ANY) {
                     R val, der;
                     const int j = (int)(e[q] & kIndexMask);
                     spline_r(T.f[B.type[s][j]], B.coef, r, val, der);
                     rho += val;
                 } else {
                     R t;
-                    const int kk = tab.interval(g, r, t);
+                    int kk = tab.interval(g, r, t);
+                    if (KIND == KIND_TYPES) kk += (int)tab.type8[e[q] & kIndexMask] * g.nint;
                     const R4 c = tab.f(kk);
                     rho += fma(t, fma(t, fma(t, c.w, c.z), c.y), c.x);
                 }
@@ -314,7 +339,7 @@ __device__ __forceinline__ R embed(const Bufs<R> &B, typename V4<R>::T *sw, int 
 //   F_i  = sum_j s_ij (x_j - x_i) / r,
 // and, when ENERGY, of the pair energy and the virial (e7: pair energy, then
 // W xx yy zz xy xz yz).
-template <class R, bool MULTI, bool ENERGY, int TPA, int U, class List, class Fetch, class Tab>
+template <class R, int KIND, bool ENERGY, int TPA, int U, class List, class Fetch, class Tab>
 __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, const R (&h)[3], R rc2,
                                            int s, const int *nnb_i, int cap, int l, int ti,
                                            const typename V4<R>::T &ui, const List &list, const Fetch &fetch, R (&f)[3], R (&e7)[7],
@@ -353,7 +378,13 @@ __device__ __forceinline__ void force_lane(const Bufs<R> &B, const Launch &L, co
                 inv_r(p.r2, rinv, r);
                 const R Fpj = u[q].w;
                 R phv, phd, fdj, fdi;
-                if (MULTI) {
+                if (KIND == KIND_TYPES) {
+                    static_assert(KIND != KIND_TYPES || !ENERGY, "energies take the general kernels");
+                    R t;
+                    const int kk = tab.interval(g, r, t);
+                    tab.slopes_types(L.ntypes, g.nint, ti, (int)tab.type8[e[q] & kIndexMask], kk, t, fdi, fdj, phd);
+                    phv = (R)0;
+                } else if (KIND == KIND_ANY) {
                     const int j = (int)(e[q] & kIndexMask);
                     const int tj = B.type[s][j];
                     spline_r(T.phi[pair_index(L.ntypes, ti, tj)], B.coef, r, phv, phd);
@@ -456,7 +487,7 @@ __device__ __forceinline__ void force_block_end(const Bufs<R> &B, const Launch &
 // The atom's density and force sums over its whole list: FP32 walks the list,
 // FP64 its columns in range.  All lanes of the warp must call; `active`: the
 // lane has an atom.
-template <class R, bool MULTI, int TPA, int U, class Fetch, class Tab>
+template <class R, int KIND, int TPA, int U, class Fetch, class Tab>
 __device__ __forceinline__ R density_atom(const Bufs<R> &B, const Geom &G, const Launch &L, const R (&h)[3], R rc2, int s,
                                           int sp, int i, int l, bool active, const Fetch &fetch, const Tab &tab)
 {
@@ -472,19 +503,19 @@ __device__ __forceinline__ R density_atom(const Bufs<R> &B, const Geom &G, const
         R rho = (R)0;
         for (int k0 = 0; k0 < most; k0 += kCompactColumns) {
             const int cnt = compact_columns<TPA>(G, B.rec32[sp], uf, bound, k0, nn, l, list, buf, width);
-            rho = density_lane<R, MULTI, TPA, U>(B, h, rc2, s, &cnt, cnt, l, ui, ListCompact{buf, width}, fetch, tab,
+            rho = density_lane<R, KIND, TPA, U>(B, h, rc2, s, &cnt, cnt, l, ui, ListCompact{buf, width}, fetch, tab,
                                                  rho);
             __syncwarp();  // the buffer is free for the next columns
         }
         return rho;
     } else {
-        return active ? density_lane<R, MULTI, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, B.shadow[sp][i], list, fetch,
+        return active ? density_lane<R, KIND, TPA, U>(B, h, rc2, s, B.nnb + i, L.cap, l, B.shadow[sp][i], list, fetch,
                                                        tab)
                       : (R)0;
     }
 }
 
-template <class R, bool MULTI, bool ENERGY, int TPA, int U, class Fetch, class Tab>
+template <class R, int KIND, bool ENERGY, int TPA, int U, class Fetch, class Tab>
 __device__ __forceinline__ void force_atom(const Bufs<R> &B, const Geom &G, const Launch &L, const R (&h)[3], R rc2,
                                            int s, int sp, int i, int l, int ti, bool active, const Fetch &fetch,
                                            R (&f)[3], R (&e7)[7], const Tab &tab)
@@ -500,12 +531,12 @@ __device__ __forceinline__ void force_atom(const Bufs<R> &B, const Geom &G, cons
         const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)nn);
         for (int k0 = 0; k0 < most; k0 += kCompactColumns) {
             const int cnt = compact_columns<TPA>(G, B.rec32[sp], uf, bound, k0, nn, l, list, buf, width);
-            force_lane<R, MULTI, ENERGY, TPA, U>(B, L, h, rc2, s, &cnt, cnt, l, ti, ui, ListCompact{buf, width}, fetch, f,
+            force_lane<R, KIND, ENERGY, TPA, U>(B, L, h, rc2, s, &cnt, cnt, l, ti, ui, ListCompact{buf, width}, fetch, f,
                                                  e7, tab);
             __syncwarp();
         }
     } else if (active) {
-        force_lane<R, MULTI, ENERGY, TPA, U>(B, L, h, rc2, s, B.nnb + i, L.cap, l, ti, B.shadow[sp][i], list, fetch, f,
+        force_lane<R, KIND, ENERGY, TPA, U>(B, L, h, rc2, s, B.nnb + i, L.cap, l, ti, B.shadow[sp][i], list, fetch, f,
                                              e7, tab);
     }
 }
@@ -551,16 +582,16 @@ __device__ __forceinline__ void prefetch_warp_streams(const Bufs<R> &B, const La
 // ---- atom-parallel schedule ----
 
 // Pairs in flight per lane: the type-dependent path needs more registers a pair.
-template <class R, bool MULTI> struct PairsInFlight {
-    static constexpr int density = MULTI ? 2 : 3;
+template <class R, int KIND> struct PairsInFlight {
+    static constexpr int density = KIND == KIND_ANY ? 2 : 3;
     static constexpr int force = 2;
 };
 
-template <class R, bool MULTI, bool ENERGY, int TPA, bool TEX>
+template <class R, int KIND, bool ENERGY, int TPA, bool TEX>
 __global__ void __launch_bounds__(256) k_density(Bufs<R> B, Geom G, Launch L)
 {
     using R4 = typename V4<R>::T;
-    constexpr int U = PairsInFlight<R, MULTI>::density;
+    constexpr int U = PairsInFlight<R, KIND>::density;
     R h[3];
     load_h<R>(G, h);
     const DevState *st = B.st;
@@ -571,15 +602,15 @@ __global__ void __launch_bounds__(256) k_density(Bufs<R> B, Geom G, Launch L)
     prefetch_warp_streams<R, false>(B, L, s, i0 + (threadIdx.x >> 5) * (32 / TPA), 32 / TPA, min(st->max_nnb, L.cap));
     const int i = i0 + threadIdx.x / TPA, l = threadIdx.x % TPA;
     const bool active = i < L.n;
-    const int ti = (MULTI && active) ? B.type[s][i] : 0;
+    const int ti = (KIND != KIND_ONE && active) ? B.type[s][i] : 0;
     const R rc2 = g_rc2<R>(G);
-    const TabGlobal<R> tab{B.coef2, B.coef_f, B.coef_d};
+    const TabGlobal<R> tab(B);
     R rho;
     if constexpr (TEX)
-        rho = density_atom<R, MULTI, TPA, U>(B, G, L, h, rc2, s, sp, i, l, active,
+        rho = density_atom<R, KIND, TPA, U>(B, G, L, h, rc2, s, sp, i, l, active,
                                              TexFetch{(cudaTextureObject_t)B.tex_shadow[sp]}, tab);
     else
-        rho = density_atom<R, MULTI, TPA, U>(B, G, L, h, rc2, s, sp, i, l, active, GlobalFetch<R>{sw}, tab);
+        rho = density_atom<R, KIND, TPA, U>(B, G, L, h, rc2, s, sp, i, l, active, GlobalFetch<R>{sw}, tab);
     rho = lane_sum<TPA>(rho);
     R e_embed = (R)0;
     if (active && l == 0) e_embed = embed<R>(B, sw, i, ti, rho);
@@ -589,11 +620,11 @@ __global__ void __launch_bounds__(256) k_density(Bufs<R> B, Geom G, Launch L)
     }
 }
 
-template <class R, bool MULTI, int MODE, bool ENERGY, int TPA>
+template <class R, int KIND, int MODE, bool ENERGY, int TPA>
 __global__ void __launch_bounds__(256) k_force(Bufs<R> B, Geom G, Launch L)
 {
     using R4 = typename V4<R>::T;
-    constexpr int U = PairsInFlight<R, MULTI>::force;
+    constexpr int U = PairsInFlight<R, KIND>::force;
     R h[3];
     load_h<R>(G, h);
     const DevState *st = B.st;
@@ -604,12 +635,12 @@ __global__ void __launch_bounds__(256) k_force(Bufs<R> B, Geom G, Launch L)
     prefetch_warp_streams<R, true>(B, L, s, i0 + (threadIdx.x >> 5) * (32 / TPA), 32 / TPA, min(st->max_nnb, L.cap));
     const int i = i0 + threadIdx.x / TPA, l = threadIdx.x % TPA;
     const bool active = i < L.n;
-    const int ti = (MULTI && active) ? B.type[s][i] : 0;
+    const int ti = (KIND != KIND_ONE && active) ? B.type[s][i] : 0;
     const R rc2 = g_rc2<R>(G);
     R f[3] = {0, 0, 0};
     R e7[7] = {0, 0, 0, 0, 0, 0, 0};
-    force_atom<R, MULTI, ENERGY, TPA, U>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f, e7,
-                                         TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+    force_atom<R, KIND, ENERGY, TPA, U>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f, e7,
+                                         TabGlobal<R>(B));
 #pragma unroll
     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
     double ke = 0.0;
@@ -830,57 +861,59 @@ void force_half(const Bufs<float> &B, const Geom &G, const Launch &L)
 
 // ---- dispatch ----
 
-template <class R, bool MULTI, bool ENERGY, bool TEX>
+template <class R, int KIND, bool ENERGY, bool TEX>
 void density_tpa_fetch(const Bufs<R> &B, const Geom &G, const Launch &L)
 {
     dim3 g(L.nb_d), b(L.block_d);
     switch (L.tpa_d) {
-    case 1: k_density<R, MULTI, ENERGY, 1, TEX><<<g, b, compact_bytes<R>(L.block_d, 1), L.stream>>>(B, G, L); break;
-    case 2: k_density<R, MULTI, ENERGY, 2, TEX><<<g, b, compact_bytes<R>(L.block_d, 2), L.stream>>>(B, G, L); break;
-    case 4: k_density<R, MULTI, ENERGY, 4, TEX><<<g, b, compact_bytes<R>(L.block_d, 4), L.stream>>>(B, G, L); break;
-    default: k_density<R, MULTI, ENERGY, 8, TEX><<<g, b, compact_bytes<R>(L.block_d, 8), L.stream>>>(B, G, L); break;
+    case 1: k_density<R, KIND, ENERGY, 1, TEX><<<g, b, compact_bytes<R>(L.block_d, 1), L.stream>>>(B, G, L); break;
+    case 2: k_density<R, KIND, ENERGY, 2, TEX><<<g, b, compact_bytes<R>(L.block_d, 2), L.stream>>>(B, G, L); break;
+    case 4: k_density<R, KIND, ENERGY, 4, TEX><<<g, b, compact_bytes<R>(L.block_d, 4), L.stream>>>(B, G, L); break;
+    default: k_density<R, KIND, ENERGY, 8, TEX><<<g, b, compact_bytes<R>(L.block_d, 8), L.stream>>>(B, G, L); break;
     }
 }
 
 // Records through the texture path where both record buffers have a texture
 // object (FP32), through the load path otherwise (FP64).
-template <class R, bool MULTI, bool ENERGY>
+template <class R, int KIND, bool ENERGY>
 void density_tpa(const Bufs<R> &B, const Geom &G, const Launch &L)
 {
     if constexpr (std::is_same<R, float>::value) {
         if (B.tex_shadow[0] && B.tex_shadow[1]) {
-            density_tpa_fetch<R, MULTI, ENERGY, true>(B, G, L);
+            density_tpa_fetch<R, KIND, ENERGY, true>(B, G, L);
             return;
         }
     }
-    density_tpa_fetch<R, MULTI, ENERGY, false>(B, G, L);
+    density_tpa_fetch<R, KIND, ENERGY, false>(B, G, L);
 }
 
-template <class R, bool MULTI, int MODE, bool ENERGY>
+template <class R, int KIND, int MODE, bool ENERGY>
 void force_tpa(const Bufs<R> &B, const Geom &G, const Launch &L)
 {
     dim3 g(L.nb_f), b(L.block_f);
     switch (L.tpa_f) {
-    case 1: k_force<R, MULTI, MODE, ENERGY, 1><<<g, b, compact_bytes<R>(L.block_f, 1), L.stream>>>(B, G, L); break;
-    case 2: k_force<R, MULTI, MODE, ENERGY, 2><<<g, b, compact_bytes<R>(L.block_f, 2), L.stream>>>(B, G, L); break;
-    case 4: k_force<R, MULTI, MODE, ENERGY, 4><<<g, b, compact_bytes<R>(L.block_f, 4), L.stream>>>(B, G, L); break;
-    default: k_force<R, MULTI, MODE, ENERGY, 8><<<g, b, compact_bytes<R>(L.block_f, 8), L.stream>>>(B, G, L); break;
+    case 1: k_force<R, KIND, MODE, ENERGY, 1><<<g, b, compact_bytes<R>(L.block_f, 1), L.stream>>>(B, G, L); break;
+    case 2: k_force<R, KIND, MODE, ENERGY, 2><<<g, b, compact_bytes<R>(L.block_f, 2), L.stream>>>(B, G, L); break;
+    case 4: k_force<R, KIND, MODE, ENERGY, 4><<<g, b, compact_bytes<R>(L.block_f, 4), L.stream>>>(B, G, L); break;
+    default: k_force<R, KIND, MODE, ENERGY, 8><<<g, b, compact_bytes<R>(L.block_f, 8), L.stream>>>(B, G, L); break;
     }
 }
 
-template <class R, bool MULTI>
+template <class R, int KIND>
+void force_modes_plain(const Bufs<R> &B, const Geom &G, const Launch &L, int mode)
+{
+    if (mode == MODE_MEASURE) force_tpa<R, KIND, MODE_MEASURE, false>(B, G, L);
+    else if (mode == MODE_CLOSE) force_tpa<R, KIND, MODE_CLOSE, false>(B, G, L);
+    else force_tpa<R, KIND, MODE_CLOSE_OPEN, false>(B, G, L);
+}
+
+template <class R, int KIND>
 void force_modes(const Bufs<R> &B, const Geom &G, const Launch &L, int mode, bool energy)
 {
-    if (mode == MODE_MEASURE) {
-        if (energy) force_tpa<R, MULTI, MODE_MEASURE, true>(B, G, L);
-        else force_tpa<R, MULTI, MODE_MEASURE, false>(B, G, L);
-    } else if (mode == MODE_CLOSE) {
-        if (energy) force_tpa<R, MULTI, MODE_CLOSE, true>(B, G, L);
-        else force_tpa<R, MULTI, MODE_CLOSE, false>(B, G, L);
-    } else {
-        if (energy) force_tpa<R, MULTI, MODE_CLOSE_OPEN, true>(B, G, L);
-        else force_tpa<R, MULTI, MODE_CLOSE_OPEN, false>(B, G, L);
-    }
+    if (!energy) force_modes_plain<R, KIND>(B, G, L, mode);
+    else if (mode == MODE_MEASURE) force_tpa<R, KIND, MODE_MEASURE, true>(B, G, L);
+    else if (mode == MODE_CLOSE) force_tpa<R, KIND, MODE_CLOSE, true>(B, G, L);
+    else force_tpa<R, KIND, MODE_CLOSE_OPEN, true>(B, G, L);
 }
 
 }  // namespace
@@ -897,12 +930,15 @@ int launch_density(const Bufs<R> &B, const Geom &G, const Launch &L, bool energy
             return 2;
         }
     }
-    if (L.multi) {
-        if (energy) density_tpa<R, true, true>(B, G, L);
-        else density_tpa<R, true, false>(B, G, L);
+    // with energies several types take the general kernels (one step of a call)
+    if (L.multi == KIND_TYPES && !energy) {
+        density_tpa<R, KIND_TYPES, false>(B, G, L);
+    } else if (L.multi) {
+        if (energy) density_tpa<R, KIND_ANY, true>(B, G, L);
+        else density_tpa<R, KIND_ANY, false>(B, G, L);
     } else {
-        if (energy) density_tpa<R, false, true>(B, G, L);
-        else density_tpa<R, false, false>(B, G, L);
+        if (energy) density_tpa<R, KIND_ONE, true>(B, G, L);
+        else density_tpa<R, KIND_ONE, false>(B, G, L);
     }
     return 1;
 }
@@ -925,8 +961,9 @@ int launch_force(const Bufs<R> &B, const Geom &G, const Launch &L, int mode, boo
             return 2;
         }
     }
-    if (L.multi) force_modes<R, true>(B, G, L, mode, energy);
-    else force_modes<R, false>(B, G, L, mode, energy);
+    if (L.multi == KIND_TYPES && !energy) force_modes_plain<R, KIND_TYPES>(B, G, L, mode);
+    else if (L.multi) force_modes<R, KIND_ANY>(B, G, L, mode, energy);
+    else force_modes<R, KIND_ONE>(B, G, L, mode, energy);
     return 1;
 }
 

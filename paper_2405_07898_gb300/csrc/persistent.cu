@@ -94,11 +94,12 @@ constexpr int kListWarpPasses = 8;
 // displacement alternates between two words: the force pass of step k writes
 // word k & 1, the decision of step k + 1 reads it (the opening drift writes
 // word 1 for the decision of step 0).
-template <class R, bool MULTI, int TPA>
+template <class R, int KIND, int TPA>
 __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long long nsteps, PersistScratch *ps)
 {
     using R4 = typename V4<R>::T;
-    constexpr int UD = PairsInFlight<R, MULTI>::density, UF = PairsInFlight<R, MULTI>::force;
+    constexpr int kEnergyKind = KIND == KIND_TYPES ? KIND_ANY : KIND;  // as the graph path's last step
+    constexpr int UD = PairsInFlight<R, KIND>::density, UF = PairsInFlight<R, KIND>::force;
     DevState *st = B.st;
     unsigned *err = &st->error;
     unsigned long long target = 0;  // of the grid barriers
@@ -175,9 +176,9 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
             for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
                 const int i = tile * width + threadIdx.x / TPA;
                 const bool active = i < n;
-                const int ti = (MULTI && active) ? B.type[s][i] : 0;
-                R rho = density_atom<R, MULTI, TPA, UD>(B, G, L, h, rc2, s, sp, i, l, active, GlobalFetch<R>{sw},
-                                                        TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+                const int ti = (KIND != KIND_ONE && active) ? B.type[s][i] : 0;
+                R rho = density_atom<R, KIND, TPA, UD>(B, G, L, h, rc2, s, sp, i, l, active, GlobalFetch<R>{sw},
+                                                        TabGlobal<R>(B));
                 rho = lane_sum<TPA>(rho);
                 if (active && l == 0) e_embed += embed<R>(B, sw, i, ti, rho);
             }
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
             for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
                 const int i = tile * width + threadIdx.x / TPA;
                 const bool active = i < n;
-                const int ti = (MULTI && active) ? B.type[s][i] : 0;
+                const int ti = (KIND != KIND_ONE && active) ? B.type[s][i] : 0;
                 R f[3] = {0, 0, 0};
                 float d2 = 0.f;
                 // the integration's inputs into L1 while the pair loop runs
@@ -211,14 +212,14 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                     }
                 }
                 if (last) {
-                    force_atom<R, MULTI, true, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
-                                                        e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+                    force_atom<R, kEnergyKind, true, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
+                                                        e7, TabGlobal<R>(B));
 #pragma unroll
                     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
                     if (active) integrate<R, MODE_CLOSE, true, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
                 } else {
-                    force_atom<R, MULTI, false, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
-                                                         e7, TabGlobal<R>{B.coef2, B.coef_f, B.coef_d});
+                    force_atom<R, KIND, false, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
+                                                         e7, TabGlobal<R>(B));
 #pragma unroll
                     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
                     if (active) integrate<R, MODE_CLOSE_OPEN, false, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
@@ -253,15 +254,22 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
     }
 }
 
-template <class R, bool MULTI>
+template <class R, int KIND>
 const void *steps_kernel(int tpa)
 {
     switch (tpa) {
-    case 1: return (const void *)k_steps<R, MULTI, 1>;
-    case 2: return (const void *)k_steps<R, MULTI, 2>;
-    case 4: return (const void *)k_steps<R, MULTI, 4>;
-    default: return (const void *)k_steps<R, MULTI, 8>;
+    case 1: return (const void *)k_steps<R, KIND, 1>;
+    case 2: return (const void *)k_steps<R, KIND, 2>;
+    case 4: return (const void *)k_steps<R, KIND, 4>;
+    default: return (const void *)k_steps<R, KIND, 8>;
     }
+}
+
+template <class R>
+const void *steps_kernel_of(int multi, int tpa)
+{
+    if (multi == KIND_TYPES) return steps_kernel<R, KIND_TYPES>(tpa);
+    return multi ? steps_kernel<R, KIND_ANY>(tpa) : steps_kernel<R, KIND_ONE>(tpa);
 }
 
 }  // namespace
@@ -269,7 +277,7 @@ const void *steps_kernel(int tpa)
 template <class R>
 int persistent_grid(const Launch &L, int tpa, int block)
 {
-    const void *fn = L.multi ? steps_kernel<R, true>(tpa) : steps_kernel<R, false>(tpa);
+    const void *fn = steps_kernel_of<R>(L.multi, tpa);
     int per_sm = 0, dev = 0, nsm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, compact_bytes<R>(block, tpa)) != cudaSuccess ||
         cudaGetDevice(&dev) != cudaSuccess ||
@@ -284,7 +292,7 @@ template <class R>
 cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, const PersistSched &sched,
                          PersistScratch *ps)
 {
-    const void *fn = L.multi ? steps_kernel<R, true>(sched.tpa) : steps_kernel<R, false>(sched.tpa);
+    const void *fn = steps_kernel_of<R>(L.multi, sched.tpa);
     Bufs<R> b = B;
     Geom g = G;
     Launch l = L;

@@ -207,7 +207,9 @@ __device__ __forceinline__ void permute_atom(const Bufs<R> &B, const Geom &G, in
         B.screen[2][p] = (float)u[2];
     }
     B.id[t][p] = id;
-    B.type[t][p] = B.type[s][i];
+    const int ty = B.type[s][i];
+    B.type[t][p] = ty;
+    B.type8[p] = (uint8_t)ty;
     B.cell[p] = cell;
 }
 
