@@ -207,6 +207,16 @@ struct PersistSched {
     int tpa, block, grid;
 };
 
+// A persistent launch that evaluates a state instead of advancing it: the
+// caller's arrays are loaded (pos null: the state is there already), the list
+// is built, then density, forces, energies and virial, as the launches of
+// rebuild, density, force and reduce do.
+struct MeasureArgs {
+    int on;
+    const double *pos, *vel;
+    const int *types;
+};
+
 // Host-side launchers (rebuild.cu, pair_f32.cu, pair_f64.cu, persistent.cu).  All are asynchronous on L.stream and
 // return the number of kernels queued.
 template <class R> int launch_rebuild(const Bufs<R> &B, const Geom &G, const Launch &L);
@@ -222,7 +232,7 @@ template <class R> int launch_force(const Bufs<R> &B, const Geom &G, const Launc
 template <class R> int persistent_grid(const Launch &L, int tpa, int block);
 template <class R>
 cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, const PersistSched &sched,
-                         PersistScratch *ps);
+                         PersistScratch *ps, const MeasureArgs &measure = MeasureArgs{});
 
 template <class R> int launch_reduce(const Bufs<R> &B, const Launch &L);
 template <class R>

@@ -95,7 +95,8 @@ constexpr int kListWarpPasses = 8;
 // word k & 1, the decision of step k + 1 reads it (the opening drift writes
 // word 1 for the decision of step 0).
 template <class R, int KIND, int TPA>
-__global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long long nsteps, PersistScratch *ps)
+__global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long long nsteps, PersistScratch *ps,
+                                               MeasureArgs M)
 {
     using R4 = typename V4<R>::T;
     constexpr int kEnergyKind = KIND == KIND_TYPES ? KIND_ANY : KIND;  // as the graph path's last step
@@ -116,8 +117,13 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
     load_h<R>(G, h);
     const R rc2 = g_rc2<R>(G);
 
-    // opening kick and drift from the cached forces
-    {
+    if (M.on) {
+        // a state to evaluate: one round below, with a list build
+        if (M.pos) {
+            for (int i = gtid; i < n; i += nthreads) load_atom<R>(B, s, M.pos, M.vel, M.types, i);
+        }
+    } else {
+        // opening kick and drift from the cached forces
         float d2 = 0.f;
         for (int i = gtid; i < n; i += nthreads) d2 = fmaxf(d2, open_atom<R>(B, L, s, sp, i));
         block_max_disp(d2, &ps->maxdisp[1]);
@@ -127,11 +133,13 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
     for (long long k = 0; k < nsteps; ++k) {
         const bool last = k == nsteps - 1;
         // decision (as k_decide)
-        sp ^= 1;
-        step += 1;
-        since += 1;
+        if (!M.on) {
+            sp ^= 1;
+            step += 1;
+            since += 1;
+        }
         const float md = __uint_as_float(ld_acquire(&ps->maxdisp[(k + 1) & 1]));
-        need = (since >= L.rebuild_every) || ((double)md > L.disp2_thr);
+        need = M.on || (since >= L.rebuild_every) || ((double)md > L.disp2_thr);
         // word k & 1 was last read by the decision of step k - 1
         if (gtid == 0) ps->maxdisp[k & 1] = 0u;
 
@@ -216,7 +224,8 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
                                                         e7, TabGlobal<R>(B));
 #pragma unroll
                     for (int c = 0; c < 3; ++c) f[c] = lane_sum<TPA>(f[c]);
-                    if (active) integrate<R, MODE_CLOSE, true, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
+                    if (active && M.on) integrate<R, MODE_MEASURE, true, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
+                    else if (active) integrate<R, MODE_CLOSE, true, TPA>(B, L, s, sp, i, l, ti, f, ke, d2);
                 } else {
                     force_atom<R, KIND, false, TPA, UF>(B, G, L, h, rc2, s, sp, i, l, ti, active, GlobalFetch<R>{sw}, f,
                                                          e7, TabGlobal<R>(B));
@@ -290,7 +299,7 @@ int persistent_grid(const Launch &L, int tpa, int block)
 
 template <class R>
 cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long long nsteps, const PersistSched &sched,
-                         PersistScratch *ps)
+                         PersistScratch *ps, const MeasureArgs &measure)
 {
     const void *fn = steps_kernel_of<R>(L.multi, sched.tpa);
     Bufs<R> b = B;
@@ -298,7 +307,10 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
     Launch l = L;
     long long ns = nsteps;
     PersistScratch *p = ps;
-    void *args[] = {&b, &g, &l, &ns, &p};
+    MeasureArgs m = measure;
+    // a state is evaluated whatever the wait limit of the steps is
+    if (m.on) l.wait_ns = std::max(l.wait_ns, 1000000000ull);
+    void *args[] = {&b, &g, &l, &ns, &p, &m};
     cudaError_t e = cudaMemsetAsync(&ps->arrive, 0, sizeof(ps->arrive), L.stream);
     if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(fn, dim3(sched.grid), dim3(sched.block), args,
@@ -308,8 +320,10 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
 template int persistent_grid<float>(const Launch &, int, int);
 template int persistent_grid<double>(const Launch &, int, int);
 template cudaError_t launch_steps<float>(const Bufs<float> &, const Geom &, const Launch &, long long,
-                                         const PersistSched &, PersistScratch *);
+                                         const PersistSched &, PersistScratch *,
+                                         const MeasureArgs &);
 template cudaError_t launch_steps<double>(const Bufs<double> &, const Geom &, const Launch &, long long,
-                                          const PersistSched &, PersistScratch *);
+                                          const PersistSched &, PersistScratch *,
+                                         const MeasureArgs &);
 
 }  // namespace eammd

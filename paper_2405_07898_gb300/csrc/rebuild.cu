@@ -177,22 +177,8 @@ __global__ void __launch_bounds__(1024) k_reduce(Bufs<R> B, int nb_d, int nb_f, 
 template <class R>
 __global__ void k_load_state(Bufs<R> B, const double *pos, const double *vel, const int *types, int n)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int s = B.st->set;
-    bool finite = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double x = pos[3 * (size_t)i + a];
-        const double v = vel ? vel[3 * (size_t)i + a] : 0.0;
-        finite = finite && isfinite(x) && isfinite(v);
-        B.xr[s][a][i] = x;
-        B.d[a][i] = 0.0;
-        B.v[s][a][i] = v;
-    }
-    if (!finite) atomicOr(&B.st->error, ERR_NONFINITE);
-    B.id[s][i] = i;
-    B.type[s][i] = types[i];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) load_atom<R>(B, B.st->set, pos, vel, types, i);
 }
 
 // Device SoA (sorted) out to interleaved arrays in the caller's order.

@@ -10,6 +10,27 @@
 namespace eammd {
 namespace {
 
+// Atom i of the caller's arrays (xyz interleaved; vel may be null) into buffer
+// set s, in the caller's order.
+template <class R>
+__device__ __forceinline__ void load_atom(const Bufs<R> &B, int s, const double *pos, const double *vel, const int *types,
+                                          int i)
+{
+    bool finite = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double x = pos[3 * (size_t)i + a];
+        const double v = vel ? vel[3 * (size_t)i + a] : 0.0;
+        finite = finite && isfinite(x) && isfinite(v);
+        B.xr[s][a][i] = x;
+        B.d[a][i] = 0.0;
+        B.v[s][a][i] = v;
+    }
+    if (!finite) atomicOr(&B.st->error, ERR_NONFINITE);
+    B.id[s][i] = i;
+    B.type[s][i] = types[i];
+}
+
 // x as a float truncated toward zero, from its bits by integer operations
 // (the FP64 pipe of this GPU is narrow): 0 below 2^-126, +-inf above the
 // float range.
