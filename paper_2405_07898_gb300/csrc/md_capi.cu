@@ -1342,6 +1342,9 @@ md_status md_create(const double box[3], int64_t n, const double *pos, const dou
         L.list_block = std::min(L.block, 128);
         while (L.list_block > 32 && (n + L.list_block - 1) / L.list_block < 2 * (int64_t)nsm) L.list_block /= 2;
         L.list_block = std::max(32, L.list_block / 32 * 32);
+        int l2 = 0;
+        if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) l2 = 0;
+        L.prefetch_from = o.precision == MD_PRECISION_MIXED ? (long long)(0.8 * (double)l2) : 0;
     }
     L.pstride = std::max(1, blocks_for_host(8 * n, std::min(L.block, 64)));
     {

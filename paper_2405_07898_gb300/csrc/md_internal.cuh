@@ -190,6 +190,7 @@ struct Launch {
     cudaStream_t stream;
     cudaGraphConditionalHandle cond;  // 0 outside graph capture
     int use_cond;
+    long long prefetch_from;          // streams of a pass (bytes) from which the pair passes ask L2 for them
     unsigned long long wait_ns;       // limit of a device-side wait (grid barrier, bulk-copy barrier)
 };
 

@@ -543,8 +543,6 @@ __device__ __forceinline__ void force_atom(const Bufs<R> &B, const Geom &G, cons
 
 // ---- L2 prefetch of a warp's streams ----
 
-constexpr bool kPrefetchWarpStreams = true;
-
 __device__ __forceinline__ void prefetch_l2(const void *p)
 {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p)));
@@ -554,12 +552,19 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
 // device memory, atoms [a0, a0 + m): the list columns up to the longest list
 // of the last build and, in the force pass, the velocities, displacements
 // and reference coordinates its integration reads.  A hint: nothing waits on
-// it, and every address lies inside its array.
+// it, and every address lies inside its array.  Systems whose streams stay in
+// L2 from pass to pass (list, velocities, displacements, reference
+// coordinates and records of all atoms, in FP32 4 bytes a neighbour and 92 an
+// atom, below L.prefetch_from = 0.8 of L2) gain nothing from the hints and pay
+// for them: us a step with and without, BCC 118,638 atoms (23 MB) 44.8 and 42.5,
+// 453,962 (89 MB) 112.0 and 107.6, 574,992 (113 MB) 136.5 and 136.9, 686,000
+// (134 MB) 155.4 and 163.5; FCC 256,000 (79 MB) 129 and 123.5, 470,596 (145 MB)
+// 215.5 and 224.  The FP64 path always asks (314,928 atoms: 547 and 560).
 template <class R, bool FORCE>
 __device__ __forceinline__ void prefetch_warp_streams(const Bufs<R> &B, const Launch &L, int s, int a0, int m,
                                                       int ncol)
 {
-    if (!kPrefetchWarpStreams || a0 >= L.n) return;
+    if (a0 >= L.n || (long long)L.n * (4 * (long long)ncol + 92) < L.prefetch_from) return;
     const int lane = threadIdx.x & 31;
     for (int k = lane; k < ncol; k += 32) prefetch_l2(B.list + (size_t)k * L.ld + a0);
     if (FORCE) {
@@ -584,7 +589,9 @@ __device__ __forceinline__ void prefetch_warp_streams(const Bufs<R> &B, const La
 // Pairs in flight per lane: the type-dependent path needs more registers a pair.
 template <class R, int KIND> struct PairsInFlight {
     static constexpr int density = KIND == KIND_ANY ? 2 : 3;
-    static constexpr int force = 2;
+    // (type pairs: one, whose 64-byte row already holds more registers; 184,320
+    // atoms 35.0 us, 42.5 with two)
+    static constexpr int force = KIND == KIND_TYPES && sizeof(R) == 4 ? 1 : 2;
 };
 
 template <class R, int KIND, bool ENERGY, int TPA, bool TEX>
