@@ -264,7 +264,7 @@ md_status md_stats(md_ctx *ctx, md_stats_t *out);
 typedef struct {
     double density_ms;       /* average density (Eq. 2) kernel */
     double force_ms;         /* average force + integration (Eqs. 4, 5) kernel */
-    double rebuild_ms;       /* average full list rebuild (8 kernels) */
+    double rebuild_ms;       /* average full list rebuild */
     double step_ms;          /* average wall time of one step on the stream */
     int64_t density_launches, force_launches, rebuilds;
 } md_profile_t;

@@ -9,10 +9,10 @@
 //
 // Grid barriers: all blocks are resident (cooperative launch); a barrier is
 // an arrival counter in device memory.  A wait gives up after the wait limit
-// (md_options.wait_limit_us, 1 s by default) of %globaltimer, raises
-// ERR_TIMEOUT and every later barrier of the launch returns at once, so the
-// kernel ends within about the limit of a stuck block and the host reports
-// MD_ERR_TIMEOUT.
+// (md_options.wait_limit_us, 1 s by default) of %globaltimer and raises
+// ERR_TIMEOUT; the block leaves the kernel, and the others see the error word
+// or run into the limit themselves, so the kernel ends within about the limit
+// of a stuck block and the host reports MD_ERR_TIMEOUT.
 #include "pair_kernels.cuh"
 #include "rebuild_device.cuh"
 
