@@ -375,7 +375,7 @@ md_status measure(md_ctx *ctx, const double *pos = nullptr, const double *vel = 
         ctx->fixed_launches += 1;
         return MD_OK;
     }
-    if (pos) ctx->fixed_launches += launch_load_state<R>(B, L, pos, vel, ctx->types_orig);
+    if (pos) ctx->fixed_launches += launch_load_state<R>(B, ctx->G, L, pos, vel, ctx->types_orig);
     ctx->fixed_launches += launch_rebuild<R>(B, ctx->G, L);
     ctx->fixed_launches += launch_density<R>(B, ctx->G, L, true);
     ctx->fixed_launches += launch_force<R>(B, ctx->G, L, MODE_MEASURE, true);
@@ -578,6 +578,8 @@ md_status profile_impl(md_ctx *ctx, int64_t nsteps, double dt, md_profile_t *out
     L.cond = 0;
     md_status rc0 = read_state(ctx);
     if (rc0 != MD_OK) return rc0;
+    // no build from what a timed-out launch left (a half-filled cell grid)
+    if (ctx->st_host->error & ERR_TIMEOUT) return state_errors(ctx);
     const long long rebuilds0 = ctx->st_host->rebuilds;
     touch(ctx);
     const int64_t ne = 4 * nsteps + 2;

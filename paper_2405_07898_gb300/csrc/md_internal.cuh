@@ -237,7 +237,8 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
 
 template <class R> int launch_reduce(const Bufs<R> &B, const Launch &L);
 template <class R>
-int launch_load_state(const Bufs<R> &B, const Launch &L, const double *pos, const double *vel, const int *types);
+int launch_load_state(const Bufs<R> &B, const Geom &G, const Launch &L, const double *pos, const double *vel,
+                      const int *types);
 template <class R>
 int launch_store_state(const Bufs<R> &B, const Launch &L, double *pos, double *vel, double *force);
 

@@ -104,8 +104,9 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
     DevState *st = B.st;
     unsigned *err = &st->error;
     unsigned long long target = 0;  // of the grid barriers
-    // a launch that timed out left its phase half done: nothing runs on it
-    // until the state is set anew (the error word is cleared then)
+    // a launch that timed out left its phase half done, and a build that it
+    // had begun left its cell counts: nothing runs on it until the state is
+    // set anew (the error word is cleared then, the counts as it is loaded)
     if (__syncthreads_or((int)(ld_acquire(err) & ERR_TIMEOUT))) return;
     int s = st->set, sp = st->sp, since = st->since_build;
     long long step = st->step, rebuilds = 0;
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
         // a state to evaluate: one round below, with a list build
         if (M.pos) {
             for (int i = gtid; i < n; i += nthreads) load_atom<R>(B, s, M.pos, M.vel, M.types, i);
+            for (int c = gtid; c < G.ncells; c += nthreads) B.count[c] = 0;  // a launch that timed out leaves its counts
         }
     } else {
         // opening kick and drift from the cached forces
@@ -311,7 +313,7 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
     // a state is evaluated whatever the wait limit of the steps is
     if (m.on) l.wait_ns = std::max(l.wait_ns, 1000000000ull);
     void *args[] = {&b, &g, &l, &ns, &p, &m};
-    cudaError_t e = cudaMemsetAsync(&ps->arrive, 0, sizeof(ps->arrive), L.stream);
+    cudaError_t e = cudaMemsetAsync(ps, 0, sizeof(PersistScratch), L.stream);
     if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(fn, dim3(sched.grid), dim3(sched.block), args,
                                        compact_bytes<R>(sched.block, sched.tpa), L.stream);

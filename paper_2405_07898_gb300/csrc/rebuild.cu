@@ -173,12 +173,14 @@ __global__ void __launch_bounds__(1024) k_reduce(Bufs<R> B, int nb_d, int nb_f, 
 }
 
 // Host arrays in, device SoA out: state of md_create / md_set_state in the
-// caller's atom order (the next list build sorts it).
+// caller's atom order (the next list build sorts it).  The cell counts start
+// from zero: a single launch that timed out inside a build leaves its own.
 template <class R>
-__global__ void k_load_state(Bufs<R> B, const double *pos, const double *vel, const int *types, int n)
+__global__ void k_load_state(Bufs<R> B, const double *pos, const double *vel, const int *types, int n, int ncells)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) load_atom<R>(B, B.st->set, pos, vel, types, i);
+    for (int c = i; c < ncells; c += gridDim.x * blockDim.x) B.count[c] = 0;
 }
 
 // Device SoA (sorted) out to interleaved arrays in the caller's order.
@@ -248,9 +250,10 @@ int launch_reduce(const Bufs<R> &B, const Launch &L)
 }
 
 template <class R>
-int launch_load_state(const Bufs<R> &B, const Launch &L, const double *pos, const double *vel, const int *types)
+int launch_load_state(const Bufs<R> &B, const Geom &G, const Launch &L, const double *pos, const double *vel,
+                      const int *types)
 {
-    k_load_state<R><<<L.nblocks, L.block, 0, L.stream>>>(B, pos, vel, types, L.n);
+    k_load_state<R><<<L.nblocks, L.block, 0, L.stream>>>(B, pos, vel, types, L.n, G.ncells);
     return 1;
 }
 
@@ -266,8 +269,8 @@ int launch_store_state(const Bufs<R> &B, const Launch &L, double *pos, double *v
     template int launch_decide<R>(const Bufs<R> &, const Launch &);                             \
     template int launch_open<R>(const Bufs<R> &, const Geom &, const Launch &);                 \
     template int launch_reduce<R>(const Bufs<R> &, const Launch &);                             \
-    template int launch_load_state<R>(const Bufs<R> &, const Launch &, const double *, const double *, \
-                                      const int *);                                             \
+    template int launch_load_state<R>(const Bufs<R> &, const Geom &, const Launch &, const double *,   \
+                                      const double *, const int *);                             \
     template int launch_store_state<R>(const Bufs<R> &, const Launch &, double *, double *, double *);
 
 EAMMD_INSTANTIATE(float)
