@@ -353,15 +353,25 @@ md_status check_device_errors(md_ctx *ctx)
     return state_errors(ctx);
 }
 
-// Rebuild + density + force (no integration) + reduction at the current
-// positions, or (pos) at those loaded from device arrays in the caller's
-// order: the state after md_create / md_set_state.  Systems that step as a
-// single launch are evaluated by one too, in FP64 up to kMeasureFp64Atoms
-// (md_set_state of 2,000 atoms in FP64 71 us against 84 with a launch per
-// kernel, 6,750 114 against 102; mixed 1,024 68 against 73, 18,522 99
-// against 106, 59,582 127 against 145).
+// Whether a state is evaluated by one launch: in systems that step so, in FP64
+// up to kMeasureFp64Atoms (md_set_state of 2,000 atoms in FP64 71 us against
+// 84 with a launch per kernel, 6,750 114 against 102; mixed 1,024 68 against
+// 73, 18,522 99 against 106, 59,582 127 against 145).  measure and reevaluate
+// go the same way, so that a state gives the same bits whether md_create,
+// md_set_state or md_set_potential evaluated it (the lanes per atom of the two
+// ways, and the partition of the energy sums, may differ).
 constexpr int64_t kMeasureFp64Atoms = 4096;
 
+template <class R>
+bool evaluates_by_one_launch(const md_ctx *ctx)
+{
+    return ctx->persist.grid > 0 && (sizeof(R) == 4 || ctx->n <= kMeasureFp64Atoms);
+}
+
+// Rebuild + density + force (no integration) + reduction at the current
+// positions, or (pos) at those loaded from device arrays in the caller's
+// order: the state after md_set_state, and md_create's before its schedules
+// are chosen.
 template <class R>
 md_status measure(md_ctx *ctx, const double *pos = nullptr, const double *vel = nullptr)
 {
@@ -370,8 +380,9 @@ md_status measure(md_ctx *ctx, const double *pos = nullptr, const double *vel = 
     Launch L = ctx->L;
     L.use_cond = 0;
     L.cond = 0;
-    if (ctx->persist.grid > 0 && (sizeof(R) == 4 || ctx->n <= kMeasureFp64Atoms)) {
-        CK(launch_steps<R>(B, ctx->G, L, 1, ctx->persist, ctx->ps, MeasureArgs{1, pos, vel, ctx->types_orig}));
+    if (evaluates_by_one_launch<R>(ctx)) {
+        CK(launch_steps<R>(B, ctx->G, L, 1, ctx->persist, ctx->ps,
+                           MeasureArgs{MEASURE_REBUILD, pos, vel, ctx->types_orig}));
         ctx->fixed_launches += 1;
         return MD_OK;
     }
@@ -777,7 +788,8 @@ struct TuneChoice {
 std::mutex g_tune_mu;
 std::vector<std::pair<TuneKey, TuneChoice>> g_tune_cache;
 
-// Density and force (forces only, no integration) at the current state.
+// Density and force (forces only, no integration) at the current state, with
+// the list as it is.
 template <class R>
 md_status reevaluate(md_ctx *ctx)
 {
@@ -785,6 +797,11 @@ md_status reevaluate(md_ctx *ctx)
     const Bufs<R> &B = bufs<R>(ctx);
     Launch L = ctx->L;
     L.use_cond = 0;
+    if (evaluates_by_one_launch<R>(ctx)) {
+        CK(launch_steps<R>(B, ctx->G, L, 1, ctx->persist, ctx->ps, MeasureArgs{MEASURE_KEEP_LIST, nullptr, nullptr, nullptr}));
+        ctx->fixed_launches += 1;
+        return MD_OK;
+    }
     ctx->fixed_launches += launch_density<R>(B, ctx->G, L, true);
     ctx->fixed_launches += launch_force<R>(B, ctx->G, L, MODE_MEASURE, true);
     ctx->fixed_launches += launch_reduce<R>(B, L);
@@ -1201,7 +1218,12 @@ md_status create_impl(md_ctx *ctx, const double *pos, const double *vel, const i
         rc = autotune<R>(ctx);
         if (rc != MD_OK) return rc;
     }
-    return setup_persistent<R>(ctx);
+    rc = setup_persistent<R>(ctx);
+    if (rc != MD_OK || ctx->persist.grid == 0) return rc;
+    // the forces are those of the schedules just chosen, not of the last trial's
+    rc = reevaluate<R>(ctx);
+    if (rc != MD_OK) return rc;
+    return check_device_errors(ctx);
 }
 
 }  // namespace

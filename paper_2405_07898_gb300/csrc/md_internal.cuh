@@ -210,10 +210,11 @@ struct PersistSched {
 
 // A persistent launch that evaluates a state instead of advancing it: the
 // caller's arrays are loaded (pos null: the state is there already), the list
-// is built, then density, forces, energies and virial, as the launches of
-// rebuild, density, force and reduce do.
+// is built (MEASURE_REBUILD) or kept, then density, forces, energies and
+// virial, as the launches of rebuild, density, force and reduce do.
+enum { MEASURE_REBUILD = 1, MEASURE_KEEP_LIST = 2 };
 struct MeasureArgs {
-    int on;
+    int on;  // 0: steps
     const double *pos, *vel;
     const int *types;
 };

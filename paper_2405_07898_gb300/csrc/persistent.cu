@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
     const R rc2 = g_rc2<R>(G);
 
     if (M.on) {
-        // a state to evaluate: one round below, with a list build
+        // a state to evaluate: one round below
         if (M.pos) {
             for (int i = gtid; i < n; i += nthreads) load_atom<R>(B, s, M.pos, M.vel, M.types, i);
             for (int c = gtid; c < G.ncells; c += nthreads) B.count[c] = 0;  // a launch that timed out leaves its counts
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
             since += 1;
         }
         const float md = __uint_as_float(ld_acquire(&ps->maxdisp[(k + 1) & 1]));
-        need = M.on || (since >= L.rebuild_every) || ((double)md > L.disp2_thr);
+        need = M.on ? M.on == MEASURE_REBUILD : (since >= L.rebuild_every) || ((double)md > L.disp2_thr);
         // word k & 1 was last read by the decision of step k - 1
         if (gtid == 0) ps->maxdisp[k & 1] = 0u;
 
