@@ -212,14 +212,17 @@ struct ListCompact {
     __device__ __forceinline__ uint32_t operator()(int k) const { return p[k * width]; }
 };
 
-// Upper bound of r_cut^2 in FP32 for the atom at u: twice the rounding bound
-// of r^2 from FP32 records of this size (a partner in range is at most a
-// shift and r_cut farther from its cell's centre).
+// Upper bound of r_cut^2 in FP32 for the atom at u: with m the sum of the
+// records' sizes (a partner in range is at most a shift and r_cut farther from
+// its cell's centre), the pair vector is rounded by at most d = 2 m 2^-24 and
+// r^2 by 2 r d + d^2; the margin is 2.5 times that and more, so that no pair in
+// range is missed however far outside an open box.
 __device__ __forceinline__ float compact_bound(const Geom &G, const float4 &u)
 {
     const float rc = sqrtf(G.rc2_f);
     const float m = fabsf(u.x) + fabsf(u.y) + fabsf(u.z) + 2.f * (G.h_f[0] + G.h_f[1] + G.h_f[2]) + 6.f * rc;
-    return G.rc2_f + 0x1p-24f * (10.f * rc * m + 16.f * G.rc2_f);
+    const float s = 0x1p-24f * m;
+    return G.rc2_f + (s * (10.f * rc + 16.f * s) + 0x1p-20f * G.rc2_f);
 }
 
 // Entries of columns [k0, min(k0 + kCompactColumns, nn)) of the lane's atom
@@ -248,7 +251,7 @@ __device__ __forceinline__ int compact_columns(const Geom &G, const float4 *rec,
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const PairIn<float> p = pair_vector<float>(ui, u[q], entry_shift<float>(e[q], h));
-            const bool in = (k + l + q * TPA < k1) && p.r2 < bound;
+            const bool in = (k + l + q * TPA < k1) && !(p.r2 > bound);  // (an overflow too)
             if (TPA == 1) {
                 if (in) buf[cnt * width] = e[q];
                 cnt += in ? 1 : 0;

@@ -316,16 +316,22 @@ __device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c)
 }
 
 // Half-width of the band around r_list^2 inside which FP32 does not decide,
-// for the atom at (x, y, z) of the screen: twice the bound of the rounding of
-// r^2 from coordinates of this size (a partner in the list is at most
-// r_list farther out; an image shift adds the box edge).  An atom far beyond
-// an open edge has a wide band, so its list stays exact.
+// for the atom at (x, y, z) of the screen.  With s the sum of the coordinates'
+// sizes (a partner in the list is at most r_list farther out; an image shift
+// adds the box edge), the pair vector is rounded by at most d = 3 s 2^-24, and
+// r^2 by 2 r d + d^2; the band is 1.7 times that, and 16 r_list^2 2^-24 for the
+// sum of squares.  An atom far beyond an open edge has a wide band, so its list
+// stays exact (up to 1e24 Angstrom, where the band overflows).  x has one
+// origin for the whole box, so the band also grows with the box's x edge (about
+// 0.2 exact tests an atom at 10,000 Angstrom, 2 at 100,000): the price of a row
+// of cells in one run.
 __device__ __forceinline__ float screen_margin(const Geom &G, float x, float y, float z)
 {
     const float rl = sqrtf(G.rl2_f);
     const float ex = fabsf(x) + G.box_f[0] + 2.f * rl;
     const float ey = fabsf(y) + 2.f * G.h_f[1] + 2.f * rl, ez = fabsf(z) + 2.f * G.h_f[2] + 2.f * rl;
-    return 0x1p-24f * (10.f * rl * (ex + ey + ez) + 16.f * G.rl2_f);
+    const float s = 0x1p-24f * (ex + ey + ez);
+    return s * (10.f * rl + 16.f * s) + 0x1p-20f * G.rl2_f;
 }
 
 // Verlet list of atom p: the atoms of the 27 surrounding cells (in stencil
