@@ -311,10 +311,11 @@ bool grow_list(md_ctx *ctx, int cap)
     drop_graphs(ctx);  // captured kernels hold the old list pointer
     uint32_t *nl = nullptr;
     if (!alloc_n(ctx, nl, (size_t)cap * ctx->L.ld)) return false;
-    // the old block stays owned by the context until md_destroy
+    // the old block stays owned by the context until md_destroy; until the next
+    // build the new one holds nobody's list
     B.list = nl;
     ctx->L.cap = cap;
-    return true;
+    return cudaMemsetAsync(B.nnb, 0, sizeof(int) * (size_t)ctx->n, ctx->stream) == cudaSuccess;
 }
 
 // The device state into st_host, after the work queued so far: the copy goes
@@ -1116,7 +1117,11 @@ md_status adjoint_setup(md_ctx *ctx)
 
 md_status force_match_impl(md_ctx *ctx, const double *f_ref, double e_ref, double w, double *loss, double *grad)
 {
-    md_status rc = adjoint_setup(ctx);
+    // errors first, so that nothing follows a list that was not built; after
+    // md_set_state or md_set_potential the flags are on the host already
+    md_status rc = ctx->st_current ? state_errors(ctx) : check_device_errors(ctx);
+    if (rc != MD_OK) return rc;
+    rc = adjoint_setup(ctx);
     if (rc != MD_OK) return rc;
     const size_t n = (size_t)ctx->n;
     CK(cudaMemcpyAsync(ctx->stage, f_ref, 3 * n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
@@ -1150,19 +1155,13 @@ md_status force_match_impl(md_ctx *ctx, const double *f_ref, double e_ref, doubl
     Launch L = ctx->L;
     ctx->fixed_launches += launch_adjoint(ctx->Bd, ctx->G, L, a);
     CK(cudaGetLastError());
-    // one wait for the energy, the error flags, |g|^2 and the gradient: the
-    // kernels take the energy from the device state
+    // one wait for |g|^2 and the gradient
     double *out = ctx->adj_host;
-    if (!ctx->st_current)
-        CK(cudaMemcpyAsync(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(out, ctx->adj_sq, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if (grad)
         CK(cudaMemcpyAsync(out + 1, ctx->adj_kg, sizeof(double) * (size_t)ctx->adj_nknots, cudaMemcpyDeviceToHost,
                            ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->st_current = true;
-    rc = state_errors(ctx);
-    if (rc != MD_OK) return rc;
     const double E = ctx->st_host->e_embed + ctx->st_host->e_pair, sq = out[0];
     if (grad) memcpy(grad, out + 1, sizeof(double) * (size_t)ctx->adj_nknots);
     if (loss) *loss = (E - e_ref) * (E - e_ref) / (double)n + w * sq;
