@@ -995,6 +995,9 @@ md_status setup_persistent(md_ctx *ctx)
     Launch L = ctx->L;
     L.dt = 0.0;
     for (int t = 0; t < ctx->ntypes; ++t) L.half_kick[t] = 0.0;
+    // the caller's wait limit is for steps: trials that it ended early would
+    // be timed as fast ones, and the choice is kept for other contexts
+    L.wait_ns = std::max(L.wait_ns, kLeastWaitNs);
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));

@@ -213,6 +213,8 @@ struct PersistSched {
 // is built (MEASURE_REBUILD) or kept, then density, forces, energies and
 // virial, as the launches of rebuild, density, force and reduce do.
 enum { MEASURE_REBUILD = 1, MEASURE_KEEP_LIST = 2 };
+// Least wait limit of launches that are not the caller's steps.
+constexpr unsigned long long kLeastWaitNs = 1000000000ull;
 struct MeasureArgs {
     int on;  // 0: steps
     const double *pos, *vel;

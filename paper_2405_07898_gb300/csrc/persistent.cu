@@ -311,7 +311,7 @@ cudaError_t launch_steps(const Bufs<R> &B, const Geom &G, const Launch &L, long 
     PersistScratch *p = ps;
     MeasureArgs m = measure;
     // a state is evaluated whatever the wait limit of the steps is
-    if (m.on) l.wait_ns = std::max(l.wait_ns, 1000000000ull);
+    if (m.on) l.wait_ns = std::max(l.wait_ns, kLeastWaitNs);
     void *args[] = {&b, &g, &l, &ns, &p, &m};
     cudaError_t e = cudaMemsetAsync(ps, 0, sizeof(PersistScratch), L.stream);
     if (e != cudaSuccess) return e;
