@@ -349,7 +349,8 @@ typedef struct {
 typedef struct {
     int32_t replicas, blocks, threads_per_block, list_capacity;
     int64_t atoms, steps, rebuilds, kernel_launches;
-    int32_t max_neighbors, reserved;
+    int32_t max_neighbors;
+    int32_t blocks_per_replica; /* blocks that share a replica (a cluster where more than 1) */
 } md_batch_info_t;
 
 /* pots: npot single-type potentials whose f and phi share a knot grid
@@ -373,6 +374,14 @@ md_status md_batch_energy(md_batch *b, double *pe, double *ke);
 md_status md_batch_get_state(md_batch *b, int32_t r, double *pos, double *vel, double *force);
 
 md_status md_batch_info(md_batch *b, md_batch_info_t *out);
+
+/* The shape of the batch's launches from here on: 1..5 as
+ * md_options.batch_schedule, 6, 7 and 8 clusters of 2, 4 and 8 blocks of 1,024
+ * threads per replica, 0 the one that md_batch_create chose.  Positions,
+ * velocities and forces do not depend on it; energies do through the partition
+ * of their sums only.  Waits for queued work.  Errors: MD_ERR_ARG (no such
+ * shape), MD_ERR_CUDA (it cannot be resident; the shape stays as it was). */
+md_status md_batch_set_schedule(md_batch *b, int32_t schedule);
 const char *md_batch_last_error(const md_batch *b);
 void md_batch_destroy(md_batch *b);
 

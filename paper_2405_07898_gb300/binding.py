@@ -31,7 +31,7 @@ EXPORTS = ("md_options_default", "md_create", "md_step", "md_sync", "md_energy",
            "md_virial", "md_get_state", "md_set_state", "md_neighbors", "md_cells", "md_stats",
            "md_profile", "md_last_error", "md_destroy", "md_bin_cells_noalloc", "md_set_potential",
            "md_force_match", "md_batch_create", "md_batch_step", "md_batch_energy", "md_batch_get_state",
-           "md_batch_info", "md_batch_last_error", "md_batch_destroy")
+           "md_batch_info", "md_batch_set_schedule", "md_batch_last_error", "md_batch_destroy")
 
 ALLOC_FN = C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p)
 FREE_FN = C.CFUNCTYPE(None, C.c_void_p, C.c_void_p)
@@ -86,7 +86,7 @@ class BatchInfo(C.Structure):
     _fields_ = [("replicas", C.c_int32), ("blocks", C.c_int32), ("threads_per_block", C.c_int32),
                 ("list_capacity", C.c_int32), ("atoms", C.c_int64), ("steps", C.c_int64),
                 ("rebuilds", C.c_int64), ("kernel_launches", C.c_int64), ("max_neighbors", C.c_int32),
-                ("reserved", C.c_int32)]
+                ("blocks_per_replica", C.c_int32)]
 
 
 class MDError(RuntimeError):
@@ -160,6 +160,8 @@ def load(build_if_missing: bool = True):
     L.md_batch_get_state.restype = C.c_int
     L.md_batch_info.argtypes = [C.c_void_p, C.POINTER(BatchInfo)]
     L.md_batch_info.restype = C.c_int
+    L.md_batch_set_schedule.argtypes = [C.c_void_p, C.c_int32]
+    L.md_batch_set_schedule.restype = C.c_int
     L.md_batch_last_error.argtypes = [C.c_void_p]
     L.md_batch_last_error.restype = C.c_char_p
     L.md_batch_destroy.argtypes = [C.c_void_p]
@@ -487,6 +489,11 @@ class MDBatch:
         i = BatchInfo()
         self._check(self._L.md_batch_info(self.h, C.byref(i)))
         return {k: getattr(i, k) for k, _ in BatchInfo._fields_}
+
+    def set_schedule(self, schedule: int):
+        """md_batch_set_schedule: 1..5 one block per replica, 6..8 clusters of
+        2, 4 and 8, 0 the shape chosen at creation."""
+        self._check(self._L.md_batch_set_schedule(self.h, int(schedule)))
 
     def close(self):
         if getattr(self, "h", None):

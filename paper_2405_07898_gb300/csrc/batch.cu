@@ -352,7 +352,8 @@ struct md_batch {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int grid = 0;
-    int schedule = 0;
+    int schedule = 0;               // index into kSchedules
+    int chosen = 0;                 // that of md_batch_create
     double *stage = nullptr;
     int max_n = 0;
     long long launches = 0;
@@ -453,6 +454,15 @@ void batch_config(int sched, int grid, cudaStream_t stream, cudaLaunchConfig_t &
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
     }
+}
+
+void batch_drop_graphs(md_batch *b)
+{
+    for (auto &g : b->graphs) {
+        cudaGraphExecDestroy(g.e);
+        cudaGraphDestroy(g.g);
+    }
+    b->graphs.clear();
 }
 
 // Blocks of the launch: as many teams as can be resident, at most one per
@@ -871,6 +881,7 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
         md_batch_destroy(b);
         return rc;
     }
+    b->chosen = b->schedule;
     // rebuild counters start after the initial build
     for (int r = 0; r < nrep; ++r) b->st_host[r].rebuilds = 0;
     b->st_current = false;
@@ -968,11 +979,27 @@ md_status md_batch_info(md_batch *b, md_batch_info_t *out)
     out->threads_per_block = kSchedules[b->schedule].block;
     out->list_capacity = b->cap;
     out->kernel_launches = b->launches;
+    out->blocks_per_replica = kSchedules[b->schedule].team;
     for (int r = 0; r < b->nrep; ++r) {
         out->rebuilds += b->st_host[r].rebuilds;
         out->max_neighbors = std::max(out->max_neighbors, b->st_host[r].max_nnb);
         out->steps = std::max<int64_t>(out->steps, b->st_host[r].step);
     }
+    return MD_OK;
+}
+
+md_status md_batch_set_schedule(md_batch *b, int32_t schedule)
+{
+    if (!b) return MD_ERR_ARG;
+    if (schedule < 0 || schedule > kNumSchedules) return b->fail(MD_ERR_ARG, "schedule must be 0..8");
+    const int sched = schedule == 0 ? b->chosen : schedule - 1;
+    const int grid = batch_grid(sched, b->nrep);
+    if (grid <= 0) return b->fail(MD_ERR_CUDA, "the launch shape cannot be resident");
+    if (sched == b->schedule) return MD_OK;
+    BCK(cudaStreamSynchronize(b->stream));
+    batch_drop_graphs(b);  // captured with the other shape
+    b->schedule = sched;
+    b->grid = grid;
     return MD_OK;
 }
 
@@ -982,10 +1009,7 @@ void md_batch_destroy(md_batch *b)
 {
     if (!b) return;
     if (b->stream) cudaStreamSynchronize(b->stream);
-    for (auto &g : b->graphs) {
-        cudaGraphExecDestroy(g.e);
-        cudaGraphDestroy(g.g);
-    }
+    batch_drop_graphs(b);
     for (void *p : b->allocs) {
         if (b->opt.free) b->opt.free(p, b->opt.alloc_ctx);
         else cudaFree(p);
