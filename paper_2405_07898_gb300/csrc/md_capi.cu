@@ -55,6 +55,9 @@ bool spline_ok(const md_spline &s)
     return true;
 }
 
+// Most bytes that the rows per type pair of an alloy may take.
+constexpr size_t kPairRowsMax = 256u << 20;
+
 // Largest system whose state is stored straight into pinned host memory.
 constexpr int64_t kHostStageAtoms = 8192;
 
@@ -732,13 +735,19 @@ md_status build_tables(md_ctx *ctx, const md_potential *pot, std::vector<double>
             for (int c = 0; c < 4; ++c) rows2.push_back(rows[4 * ((size_t)tab.f[0].offset + k) + c]);
     }
     // several types whose f and phi all share a knot grid: per type pair the
-    // rows of the three derivatives that its force needs, then the f rows
-    bool shared = pot->ntypes > 1;
+    // rows of the three derivatives that its force needs, then the f rows.
+    // Faster than the general kernels at every size measured (184,320 atoms in
+    // FP32, us a step: 2 types of 400 knots 64 against 86, 8 of 2,000 75 against
+    // 112, 8 of 40,000, 92 MB of rows, 81 against 122), but the rows grow with
+    // the square of the types: beyond kPairRowsMax the general kernels, which
+    // need no copy, so that no table is refused for want of memory.
+    bool shared = pot->ntypes > 1 && (size_t)npair * (size_t)(f0.n - 1) * 16 * sizeof(R) <= kPairRowsMax;
     auto same = [&](const md_spline &a) { return a.n == f0.n && a.x0 == f0.x0 && a.dx == f0.dx; };
     for (int t = 0; t < pot->ntypes; ++t) shared = shared && same(pot->f[t]);
     for (int q = 0; q < npair; ++q) shared = shared && same(pot->phi[q]);
     if (shared) {
         tab.fused = 2;
+        rows2.reserve((16 * (size_t)npair + 4 * (size_t)pot->ntypes) * (size_t)(f0.n - 1));
         tab.fphi = tab.f[0];
         tab.fphi.offset = 0;
         for (int a = 0, q = 0; a < pot->ntypes; ++a)
