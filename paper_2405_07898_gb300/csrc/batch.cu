@@ -39,6 +39,9 @@ namespace eammd {
 namespace {
 
 constexpr int kMaxTeam = 8;  // blocks of a team
+// Largest replica whose state is read through pinned memory (4.7 MB); larger
+// ones are copied straight into the caller's arrays.
+constexpr int kBatchStageAtoms = 65536;
 constexpr int kBatchDensityPairs = 4, kBatchForcePairs = 2;  // pairs in flight per lane
 
 // A replica: its view of the arrays, geometry and constants (B.st is its
@@ -346,7 +349,7 @@ struct md_batch {
     bool st_current = false;        // st_host holds the device's states, st_status what they say
     md_status st_status = MD_OK;
     std::string st_message;
-    double *host_stage = nullptr;   // pinned: positions, velocities, forces of one replica
+    double *host_stage = nullptr;   // pinned: positions, velocities, forces of one replica (kBatchStageAtoms)
     std::vector<void *> allocs;
     md_options opt{};
     cudaStream_t stream = nullptr;
@@ -785,7 +788,8 @@ md_status md_batch_create(int32_t nrep, const md_replica *reps, int32_t npot, co
     for (int s = 0; s < 2 && ce == cudaSuccess; ++s) ce = cudaMemset(B.type[s], 0, sizeof(int) * N);
     for (int a = 0; a < 3 && ce == cudaSuccess; ++a) ce = cudaMemset(B.d[a], 0, sizeof(double) * N);
     if (ce == cudaSuccess) ce = cudaMallocHost((void **)&b->st_host, sizeof(DevState) * nrep);
-    if (ce == cudaSuccess) ce = cudaMallocHost((void **)&b->host_stage, sizeof(double) * 9 * (size_t)b->max_n);
+    if (ce == cudaSuccess)
+        ce = cudaMallocHost((void **)&b->host_stage, sizeof(double) * 9 * (size_t)std::min(b->max_n, kBatchStageAtoms));
     // the replicas' states, caller order within each replica
     {
         std::vector<double> x(N, 0.0);
@@ -960,6 +964,13 @@ md_status md_batch_get_state(md_batch *b, int32_t r, double *pos, double *vel, d
     k_batch_store<<<(int)((n + 255) / 256), 256, 0, b->stream>>>(b->rep_dev, r, at[0], at[1], at[2]);
     b->launches += 1;
     BCK(cudaGetLastError());
+    if (n > (size_t)kBatchStageAtoms) {
+        for (int k = 0; k < 3; ++k)
+            if (out[k])
+                BCK(cudaMemcpyAsync(out[k], at[k], sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, b->stream));
+        BCK(cudaStreamSynchronize(b->stream));
+        return MD_OK;
+    }
     BCK(cudaMemcpyAsync(b->host_stage, b->stage, sizeof(double) * len, cudaMemcpyDeviceToHost, b->stream));
     BCK(cudaStreamSynchronize(b->stream));
     for (int k = 0; k < 3; ++k)
