@@ -796,6 +796,9 @@ struct TuneChoice {
     PassSched d, f;
 };
 std::mutex g_tune_mu;
+// Entries of either cache; shapes beyond are timed at each creation (list
+// capacities are the caller's, so their number has no bound of its own).
+constexpr size_t kScheduleCacheMax = 256;
 std::vector<std::pair<TuneKey, TuneChoice>> g_tune_cache;
 
 // Density and force (forces only, no integration) at the current state, with
@@ -906,7 +909,7 @@ md_status autotune(md_ctx *ctx)
     const TuneChoice choice{cand[cd], cand[cf]};
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune_cache.push_back({key, choice});
+        if (g_tune_cache.size() < kScheduleCacheMax) g_tune_cache.push_back({key, choice});
     }
     set_sched(ctx, choice.d, choice.f);
     // forces and energies of the state under the chosen schedule
@@ -932,7 +935,6 @@ struct PersistKey {
     }
 };
 std::vector<std::pair<PersistKey, PersistSched>> g_persist_cache;  // under g_tune_mu
-constexpr size_t kPersistCacheMax = 256;
 
 // The persistent step launch: a cooperative grid of as many blocks as are
 // resident.  Lanes per atom come from the options, else every feasible
@@ -1035,7 +1037,7 @@ md_status setup_persistent(md_ctx *ctx)
     ctx->persist = cand[best_i];
     if (timed) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        if (g_persist_cache.size() < kPersistCacheMax) g_persist_cache.push_back({key, ctx->persist});
+        if (g_persist_cache.size() < kScheduleCacheMax) g_persist_cache.push_back({key, ctx->persist});
     }
     return check_device_errors(ctx);
 }
