@@ -347,6 +347,7 @@ struct md_batch {
     DevState *st = nullptr;         // one per replica
     DevState *st_host = nullptr;    // pinned
     bool st_current = false;        // st_host holds the device's states, st_status what they say
+    bool replayable = false;        // steps were captured by the caller: the states are read at every call
     md_status st_status = MD_OK;
     std::string st_message;
     double *host_stage = nullptr;   // pinned: positions, velocities, forces of one replica (kBatchStageAtoms)
@@ -515,7 +516,7 @@ md_status batch_sync(md_batch *b)
         BCK(cudaMemcpyAsync(b->st_host, b->st, sizeof(DevState) * b->nrep, cudaMemcpyDeviceToHost, b->stream));
     BCK(cudaStreamSynchronize(b->stream));
     if (!b->st_current) {
-        b->st_current = true;
+        b->st_current = !b->replayable;
         b->st_status = MD_OK;
         b->st_message.clear();
         for (int r = 0; r < b->nrep; ++r) {
@@ -902,6 +903,7 @@ md_status md_batch_step(md_batch *b, int64_t nsteps, double dt)
     if (!b) return MD_ERR_ARG;
     if (nsteps < 0 || nsteps > (int64_t)1 << 30 || !std::isfinite(dt)) return b->fail(MD_ERR_ARG, "bad nsteps or dt");
     if (nsteps == 0) return MD_OK;
+    b->replayable = b->replayable || is_capturing(b->stream);
     if (!b->opt.use_graphs) return batch_launch(b, BATCH_RUN, (int)nsteps, dt);
     for (auto &g : b->graphs)
         if (g.nsteps == (int)nsteps && g.dt == dt) {

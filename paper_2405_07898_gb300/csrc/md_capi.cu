@@ -89,6 +89,7 @@ struct md_ctx {
     DevState *st = nullptr;
     DevState *st_host = nullptr;  // pinned
     bool st_current = false;      // st_host is the device state (read_state, touch)
+    bool replayable = false;      // work was queued under stream capture: st_host is never taken as current
     double *host_stage = nullptr; // pinned, kHostStageAtoms or fewer: AoS pos, vel, force
     double *stage = nullptr;      // 9 n doubles: AoS pos, vel, force
     int *types_orig = nullptr;
@@ -330,12 +331,18 @@ md_status read_state(md_ctx *ctx)
     if (!ctx->st_current)
         CK(cudaMemcpyAsync(ctx->st_host, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->st_current = true;
+    ctx->st_current = !ctx->replayable;
     return MD_OK;
 }
 
-// To be called wherever kernels or copies that write the device state are queued.
-void touch(md_ctx *ctx) { ctx->st_current = false; }
+// To be called wherever kernels or copies that write the device state are
+// queued.  What is queued under a caller's stream capture runs whenever the
+// caller replays the graph: from then on every reading call copies the state.
+void touch(md_ctx *ctx)
+{
+    ctx->st_current = false;
+    ctx->replayable = ctx->replayable || is_capturing(ctx->stream);
+}
 
 // The error flags of the device state last read into st_host.
 md_status state_errors(md_ctx *ctx)

@@ -221,6 +221,13 @@ struct MeasureArgs {
     const int *types;
 };
 
+// Whether work queued on the stream is being captured into a caller's graph.
+inline bool is_capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone;
+}
+
 // Host-side launchers (rebuild.cu, pair_f32.cu, pair_f64.cu, persistent.cu).  All are asynchronous on L.stream and
 // return the number of kernels queued.
 template <class R> int launch_rebuild(const Bufs<R> &B, const Geom &G, const Launch &L);
