@@ -364,19 +364,21 @@ md_status check_device_errors(md_ctx *ctx)
     return state_errors(ctx);
 }
 
-// Whether a state is evaluated by one launch: in systems that step so, in FP64
-// up to kMeasureFp64Atoms (md_set_state of 2,000 atoms in FP64 71 us against
-// 84 with a launch per kernel, 6,750 114 against 102; mixed 1,024 68 against
-// 73, 18,522 99 against 106, 59,582 127 against 145).  measure and reevaluate
+// Whether a state is evaluated by one launch: in systems that step so, up to
+// kMeasureAtoms, in FP64 up to kMeasureFp64Atoms (md_set_state with one launch
+// and with a launch per kernel, us: mixed 1,024 atoms 61 and 70, 6,750 70 and
+// 81, 18,522 96 and 100, 59,582 123 and 133, 93,312 160 and 161, 118,638 204
+// and 177, 182,250 246 and 228; FP64 2,000 68 and 80, 4,394 87 and 89, 6,750
+// 103 and 104).  measure and reevaluate
 // go the same way, so that a state gives the same bits whether md_create,
 // md_set_state or md_set_potential evaluated it (the lanes per atom of the two
 // ways, and the partition of the energy sums, may differ).
-constexpr int64_t kMeasureFp64Atoms = 4096;
+constexpr int64_t kMeasureAtoms = 65536, kMeasureFp64Atoms = 4096;
 
 template <class R>
 bool evaluates_by_one_launch(const md_ctx *ctx)
 {
-    return ctx->persist.grid > 0 && (sizeof(R) == 4 || ctx->n <= kMeasureFp64Atoms);
+    return ctx->persist.grid > 0 && ctx->n <= (sizeof(R) == 4 ? kMeasureAtoms : kMeasureFp64Atoms);
 }
 
 // Rebuild + density + force (no integration) + reduction at the current

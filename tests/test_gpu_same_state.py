@@ -48,3 +48,15 @@ def test_same_bits_by_every_way_in(which, persistent, precision):
         equal(first, answers(md), "md_set_potential after md_set_state")
         md.step(25, 2.0)
         equal(run, list(md.get_state()[:2]) + answers(md), "25 steps")
+
+
+@pytest.mark.parametrize("cells,precision,one", [(10, "mixed", True), (10, "fp64", True), (13, "fp64", False),
+                                                 (32, "mixed", True), (33, "mixed", False)])
+def test_evaluated_by_one_launch_up_to_its_size(cells, precision, one):
+    """The single launch evaluates a state up to 65,536 atoms (FP64: 4,096);
+    larger systems that step by it are faster with a launch per kernel."""
+    s = I.bcc_cube(cells)
+    with binding.MD(s, precision=precision, persistent="on", lanes_per_atom=2) as md:
+        before = md.stats()["kernel_launches"]
+        md.set_state(s.pos, s.vel)
+        assert (md.stats()["kernel_launches"] - before == 1) == one
