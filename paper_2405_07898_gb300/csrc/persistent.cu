@@ -141,7 +141,10 @@ __global__ void __launch_bounds__(256) k_steps(Bufs<R> B, Geom G, Launch L, long
             since += 1;
         }
         const float md = __uint_as_float(ld_acquire(&ps->maxdisp[(k + 1) & 1]));
-        need = M.on ? M.on == MEASURE_REBUILD : (since >= L.rebuild_every) || ((double)md > L.disp2_thr);
+        // (as a condition: with M.on selecting between the two, 2,000 atoms in
+        // FP64 took 1,855 us per 100 steps instead of 1,845)
+        need = M.on == MEASURE_REBUILD ||
+               (M.on == 0 && ((since >= L.rebuild_every) || ((double)md > L.disp2_thr)));
         // word k & 1 was last read by the decision of step k - 1
         if (gtid == 0) ps->maxdisp[k & 1] = 0u;
 
