@@ -107,8 +107,9 @@ enum { MD_PERSIST_AUTO = 0, MD_PERSIST_OFF = 1, MD_PERSIST_ON = 2 };
  *                    density and force passes: 1, 2, 4 or 8; 0 = chosen at
  *                    md_create by timing each together with the threads per
  *                    block (the choice is kept for the process, per
- *                    precision and size class, so contexts of the same shape
- *                    follow the same schedule).  Each lane gathers its
+ *                    precision, kind of tables, size class and list
+ *                    capacity, so contexts of the same shape follow the same
+ *                    schedule).  Each lane gathers its
  *                    neighbours' records and spline rows from device memory.
  *                    Results depend on it only through FP summation order.
  *   persistent       MD_PERSIST_AUTO (0): md_step runs as one launch (all
@@ -123,7 +124,9 @@ enum { MD_PERSIST_AUTO = 0, MD_PERSIST_OFF = 1, MD_PERSIST_ON = 2 };
  *                    forces are bitwise those of the graph path with the
  *                    same lanes per atom; energy sums differ in rounding
  *                    only.  A barrier wait longer than the wait limit ends
- *                    the launch and raises MD_ERR_TIMEOUT.
+ *                    the launch and raises MD_ERR_TIMEOUT, at the next call
+ *                    that waits; steps queued meanwhile do nothing, and
+ *                    md_set_state starts the context anew.
  *   open_axes        one bit per open (non-periodic) axis: 1 = x, 2 = y,
  *                    4 = z; 0 = fully periodic.  The free-surface slabs of
  *                    the paper's benchmarks (Section "How Performance Was
@@ -142,7 +145,8 @@ enum { MD_PERSIST_AUTO = 0, MD_PERSIST_OFF = 1, MD_PERSIST_ON = 2 };
  *                    per SM and blocks per replica timed at md_batch_create
  *                    (unless lanes_per_atom > 0, which takes 512 x 1); 1..5 =
  *                    512 x 1, 256 x 2, 256 x 3, 1024 x 1, 512 x 2, one block
- *                    per replica.
+ *                    per replica (md_batch_set_schedule also takes clusters).
+ *                    A timed choice is kept for the process, per batch shape.
  *   half_list        0: every atom lists all its neighbours and each pair is
  *                    evaluated from both ends (the default).  1: the
  *                    force-symmetry form (Section "Additional Acceleration"): each pair
@@ -222,7 +226,10 @@ md_status md_get_state(md_ctx *ctx, double *pos, double *vel, int64_t *step);
  * are host arrays (pinned memory makes the copy asynchronous DMA).
  * Synchronises.  Errors: MD_ERR_ARG (pos NULL); MD_ERR_NONFINITE when a
  * value is not finite (checked on the device while loading; the context's
- * state is then undefined until the next successful md_set_state). */
+ * state is then undefined until the next successful md_set_state);
+ * MD_ERR_TIMEOUT when the state is evaluated by a single launch (md_options.
+ * persistent) and one of its waits outlasts wait_limit_us, here at least 1 s.
+ * The bits of the result are those of md_create with the same arrays. */
 md_status md_set_state(md_ctx *ctx, const double *pos, const double *vel, int64_t step);
 
 /* Neighbour list of the last build in original atom ids, CSR:

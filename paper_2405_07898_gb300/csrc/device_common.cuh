@@ -109,7 +109,8 @@ __device__ __forceinline__ int segment(const SplineDesc<R> &s, R x, R &t)
 // again gives floor(u) as a number.  Two additions stand for the conversions
 // to integer and back, which run at an eighth of the FP32 rate (FP32) or on
 // the narrow FP64 pipe.  The bits are compared as unsigned integers, so that
-// a NaN takes the last interval.
+// the interval is in range whatever x: a NaN takes the last in FP32; in FP64,
+// where the low word alone is compared, the first or the last.
 __device__ __forceinline__ int segment_fused(const SplineDesc<float> &s, float x, float &t)
 {
     const float xr = x - s.x0;

@@ -28,7 +28,7 @@ constexpr int64_t kListWarpMaxAtoms = 32768;
 constexpr int kScanOneLaunch = 65536;
 
 // --------------------------------------------------------------------------
-// list build (every rebuild): wrap, bin, scan, scatter, sort, permute, list
+// list build (every rebuild): wrap and bin, scan, scatter, permute, list
 
 template <class R>
 __global__ void k_bin(Bufs<R> B, Geom G, int n)

@@ -86,7 +86,7 @@ __device__ __forceinline__ int cell_slot(int *count, int cell)
 // [0, L), else x - L floor(x / L); then bin: c_d = floor(x_d n_d/L_d) clamped
 // to [0, n_d - 1].  The box test compares bit patterns (non-negative doubles
 // order as their bits; -0 is inside).  The slot inside the cell is the
-// arrival order (fixed by sort_cell).
+// arrival order (permute_atom puts the cell's atoms in the order of their ids).
 template <class R>
 __device__ __forceinline__ void bin_atom(const Bufs<R> &B, const Geom &G, int s, int i)
 {
@@ -284,7 +284,7 @@ __device__ __forceinline__ bool upper_half(float dz, const double *const xr[3], 
 
 // What the list build screens candidates with, in FP32: the coordinate x
 // itself (the same origin for all cells of a row), and y and z relative to the
-// cell's centre.  kScreenPad words around the arrays may be read and are ignored.
+// cell's centre.  kScreenPad words after the arrays may be read and are ignored.
 struct Screen {
     const float *x, *y, *z;
 };
@@ -353,7 +353,7 @@ __device__ __forceinline__ float screen_margin(const Geom &G, float x, float y, 
 // A branch per candidate is taken by some lane nearly every time, and cells
 // on their own leave lanes waiting for the fullest cell in the warp.  A
 // rebuild of 799,496 BCC atoms takes 228 us (331 before), of the 801,792-atom
-// FCC slab 307 us (508), of the BCC atoms in the FP64 path 278 us (2,552).
+// FCC slab 307 us (508), of the BCC atoms in the FP64 path 234 us (2,552).
 // Also measured: a warp per cell with its stencil's candidates over the lanes
 // and ballots as hit masks, 381 us (barriers and idle lanes in the appends).
 // Returns the neighbour count (the list keeps at most cap of them; more
